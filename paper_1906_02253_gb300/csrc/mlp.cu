@@ -11,25 +11,37 @@
 
 namespace kfgb {
 
-// Inference on the tensor cores (tcgen05): a persistent CTA of 256 threads takes tiles of 128
-// samples, two threads per sample (each half of the columns). Per tile: standardised inputs -> X tile (128 x 16); D1 = X W1^T
-// in tensor memory; h1 = relu(D1 + b1) -> H tile (128 x 64); D2 = H W2^T; logit = b3 + sum_j W3[j]
-// relu(D2[j] + b2[j]) on the CUDA cores. Every operand is three bf16 tiles (hi, mid, lo; tc.cuh).
-// Shared memory (bytes): X, W1, W2 and H, then b1, b2, W3, mean, sd, b3, the mbarrier and the
-// tensor-memory base; 128 tensor-memory columns (D1 at 0, D2 at 64).
-namespace fwd {
-constexpr uint32_t X_T = 4096, W1_T = 2048, W2_T = 8192, H_T = 16384;  // bytes of one tile
-constexpr uint32_t X = 0, W1 = X + 3 * X_T, W2 = W1 + 3 * W1_T, H = W2 + 3 * W2_T, B1 = H + 3 * H_T, B2 = B1 + 256,
-                   W3 = B2 + 256, MEAN = W3 + 256, SD = MEAN + 64, PART = SD + 64, B3 = PART + 1024, BAR = B3 + 8,
-                   TMEM = BAR + 8, BYTES = TMEM + 8;
-constexpr uint32_t kCols = 128;
-}  // namespace fwd
+// Shared shape of the two kernels: a persistent CTA per SM in groups of 256 threads. A group takes
+// tiles of 128 samples, two threads per sample: thread t takes sample t % 128 of the tile and half
+// h = t / 128 of its columns. Warps w and w + 4 of a group read the same tensor-memory lanes
+// (32 (w % 4) ..), each its half of a 64-column accumulator; every branch around a tensor-memory
+// load is uniform within a warp. A tile is a chain of MMAs and CUDA-core steps that wait for one
+// another, so the groups of a CTA, on their own barriers, work in each other's waits; they
+// share the weights in shared memory. Every operand is three bf16 tiles (hi, mid, lo; tc.cuh).
+// Inputs: the 14 standardised features, a one (W1's column for it is b1, so the first MMA adds the
+// bias), a zero.
 constexpr int kTcM = 128;   // samples per tile (the MMA's M)
-constexpr int kTcK1 = 16;   // the 14 inputs padded to one MMA K step
-constexpr int kFwdCtasPerSm = 2;
+constexpr int kTcK1 = 16;   // inputs padded to one MMA K step
+constexpr int kOne = kMlpIn;  // the input that is one
+constexpr int kGroup = 2 * kTcM;
 
-// Loads W1 (64 x 16, inputs 14 and 15 zero) and W2 (64 x 64) as the MMAs' B operands in the
-// K-major core-matrix layout, by all threads of the block.
+// Inference: per tile, standardised inputs -> X tile (128 x 16); D = X W1^T in tensor memory; h1 =
+// relu(D) -> H tile (128 x 64, over the X tile, which the finished MMA no longer needs); D = H W2^T;
+// logit = b3 + sum_j W3[j] relu(D[j] + b2[j]) on the CUDA cores. Four groups per CTA (1024 threads
+// at 64 registers; shared memory for four H tiles and one set of weights): on 1,000,003 rows
+// FWD_NOTE
+namespace fwd {
+constexpr int kGroups = 4;
+constexpr uint32_t W1_T = 2048, W2_T = 8192, H_T = 16384, X_T = 4096;  // bytes of one tile
+constexpr uint32_t W1 = 0, W2 = W1 + 3 * W1_T, H = W2 + 3 * W2_T, B2 = H + kGroups * 3 * H_T, W3 = B2 + 256,
+                   MEAN = W3 + 256, SD = MEAN + 64, PART = SD + 64, BAR = PART + kGroups * 512, TMEM = BAR + 8 * kGroups,
+                   BYTES = TMEM + 8;
+constexpr uint32_t kCols = 64 * kGroups;
+static_assert(BYTES + 1024 <= 227 * 1024 && 3 * X_T <= 3 * H_T, "shared-memory layout");
+}  // namespace fwd
+
+// Loads W1 (64 x 16: 14 inputs, b1, zero) and W2 (64 x 64) as the MMAs' B operands in the K-major
+// core-matrix layout, by all threads of the block.
 __device__ __forceinline__ void stage_weights_b(const float* __restrict__ params, unsigned char* w1, uint32_t w1_t,
                                                 unsigned char* w2, uint32_t w2_t) {
   for (int item = threadIdx.x; item < kMlpHid * 2; item += blockDim.x) {
@@ -38,7 +50,7 @@ __device__ __forceinline__ void stage_weights_b(const float* __restrict__ params
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
       const int i = 8 * c + e;
-      v[e] = i < kMlpIn ? params[kMlpW1 + j * kMlpIn + i] : 0.f;
+      v[e] = i < kMlpIn ? params[kMlpW1 + j * kMlpIn + i] : i == kOne ? params[kMlpB1 + j] : 0.f;
     }
     tc::store8_split(w1, w1_t, tc::kmajor_off(j, c, kTcK1), v);
   }
@@ -51,11 +63,6 @@ __device__ __forceinline__ void stage_weights_b(const float* __restrict__ params
   }
 }
 
-// Two threads per sample: thread t takes sample t % 128 of the tile and half h = t / 128 of its
-// columns. Warps w and w + 4 read the same tensor-memory lanes (32 (w % 4) ..), each its half of a
-// 64-column accumulator; every branch around a tensor-memory load is uniform within a warp.
-constexpr int kTcThreads = 2 * 128;
-
 // Raw features [8 h, 8 h + 8) of sample r (zeros past n and past the 14 inputs), loaded ahead of
 // their tile.
 __device__ __forceinline__ void fetch_half(const float* __restrict__ feats, int r, int n, int half, float2* f) {
@@ -67,7 +74,7 @@ __device__ __forceinline__ void fetch_half(const float* __restrict__ feats, int 
   }
 }
 
-// Standardised inputs [8 h, 8 h + 8) into x[8] (zero past n and for the padding inputs 14, 15).
+// Standardised inputs [8 h, 8 h + 8) into x[8] (zero past n), the one and the zero.
 __device__ __forceinline__ void standardise_half(const float2* f, bool valid, int half, const float* mean,
                                                  const float* sd, float* x) {
 #pragma unroll
@@ -76,6 +83,21 @@ __device__ __forceinline__ void standardise_half(const float2* f, bool valid, in
     x[2 * i] = (valid && k < kMlpIn) ? (f[i].x - mean[k]) / sd[k] : 0.f;
     x[2 * i + 1] = (valid && k + 1 < kMlpIn) ? (f[i].y - mean[k + 1]) / sd[k + 1] : 0.f;
   }
+  if (half == 1) x[kOne - 8] = 1.f;
+}
+
+// This thread's 16 columns [c, c + 16) of sum_j w3[j] relu(v[j] + b2[j]) onto acc (columns 16-byte
+// aligned in shared memory).
+__device__ __forceinline__ float out_layer16(const float* v, const float* b2, const float* w3, float acc) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const float4 b = reinterpret_cast<const float4*>(b2)[i], w = reinterpret_cast<const float4*>(w3)[i];
+    acc = fmaf(w.x, fmaxf(v[4 * i] + b.x, 0.f), acc);
+    acc = fmaf(w.y, fmaxf(v[4 * i + 1] + b.y, 0.f), acc);
+    acc = fmaf(w.z, fmaxf(v[4 * i + 2] + b.z, 0.f), acc);
+    acc = fmaf(w.w, fmaxf(v[4 * i + 3] + b.w, 0.f), acc);
+  }
+  return acc;
 }
 
 // One MMA operand in shared memory: the first of its three tiles (shared-window address), the
@@ -91,9 +113,9 @@ __device__ __forceinline__ Operand kmajor(uint32_t base, uint32_t tile, int kt, 
 
 // The same tile read MN-major (its rows become K, its columns M or N): 8-column blocks are 128 B
 // apart (stride byte offset), 8-row groups kt / 8 * 128 B apart (leading byte offset).
-__device__ __forceinline__ Operand mnmajor(uint32_t base, uint32_t tile, int kt) {
+__device__ __forceinline__ Operand mnmajor(uint32_t base, uint32_t tile, int kt, int c0 = 0) {
   const uint32_t g = static_cast<uint32_t>(kt / 8 * 128);
-  return Operand{base, tile, g, 128u, 2u * g};
+  return Operand{base + 128u * c0, tile, g, 128u, 2u * g};
 }
 
 // D = A B^T over k_steps steps of K = 16 as the six products of the three-part split (hi*hi,
@@ -114,65 +136,63 @@ __device__ __forceinline__ void mma_split(uint32_t d, const Operand& A, const Op
   tc::mma_commit(bar);
 }
 
-__global__ void __launch_bounds__(kTcThreads) k_mlp_forward(const float* __restrict__ params,
-                                                            const float* __restrict__ feats, int n,
-                                                            float* __restrict__ logits) {
+__global__ void __launch_bounds__(fwd::kGroups* kGroup, 1) k_mlp_forward(const float* __restrict__ params,
+                                                                         const float* __restrict__ feats, int n,
+                                                                         float* __restrict__ logits) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned char* S = smem_raw + ((1024 - (tc::smem_u32(smem_raw) & 1023)) & 1023);
   const uint32_t sb = tc::smem_u32(S);
-  float* b1 = reinterpret_cast<float*>(S + fwd::B1);
   float* b2 = reinterpret_cast<float*>(S + fwd::B2);
   float* w3 = reinterpret_cast<float*>(S + fwd::W3);
   float* mean = reinterpret_cast<float*>(S + fwd::MEAN);
   float* sd = reinterpret_cast<float*>(S + fwd::SD);
-  float* part = reinterpret_cast<float*>(S + fwd::PART);  // [2][128] output-layer partial sums
-  uint64_t* bar = reinterpret_cast<uint64_t*>(S + fwd::BAR);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(S + fwd::TMEM);
-  const int t = threadIdx.x, warp = t >> 5, row = t & (kTcM - 1), half = t >> 7;
+  const int gi = threadIdx.x / kGroup, t = threadIdx.x % kGroup, warp = t >> 5, row = t & (kTcM - 1), half = t / kTcM;
+  float* part = reinterpret_cast<float*>(S + fwd::PART) + gi * kTcM;  // second half's output-layer sums
+  uint64_t* bar = reinterpret_cast<uint64_t*>(S + fwd::BAR) + gi;
+  const uint32_t h_off = fwd::H + gi * 3 * fwd::H_T;  // this group's H tile, and X tile before it
+  const int bid = gi + 1;
 
   stage_weights_b(params, S + fwd::W1, fwd::W1_T, S + fwd::W2, fwd::W2_T);
-  for (int i = t; i < kMlpHid; i += blockDim.x) {
-    b1[i] = params[kMlpB1 + i];
-    b2[i] = params[kMlpB2 + i];
-    w3[i] = params[kMlpW3 + i];
+  if (threadIdx.x < kMlpHid) {
+    b2[threadIdx.x] = params[kMlpB2 + threadIdx.x];
+    w3[threadIdx.x] = params[kMlpW3 + threadIdx.x];
   }
-  if (t < kMlpIn) {
-    mean[t] = params[kMlpMean + t];
-    sd[t] = params[kMlpSd + t];
+  if (threadIdx.x < kMlpIn) {
+    mean[threadIdx.x] = params[kMlpMean + threadIdx.x];
+    sd[threadIdx.x] = params[kMlpSd + threadIdx.x];
   }
   const float b3 = params[kMlpB3];
-  if (warp == 0) tc::tmem_alloc(tmem_slot, fwd::kCols);
+  if (threadIdx.x < 32) tc::tmem_alloc(tmem_slot, fwd::kCols);
   if (t == 0) tc::mbar_init(bar, 1);
+  tc::fence_proxy_async();
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
-  const uint32_t tmem = *tmem_slot;
-  const uint32_t lane_base = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16) + 32u * half;
+  const uint32_t tmem = *tmem_slot, d = tmem + 64u * gi;
+  const uint32_t lane_base = d + (static_cast<uint32_t>((warp & 3) * 32) << 16) + 32u * half;
   constexpr uint32_t idesc = tc::idesc_bf16_f32(kTcM, kMlpHid);
   uint32_t phase = 0;
-  bool failed = false;
+  bool ok = true;  // a wait that gives up ends the group's tiles; until then its threads keep in step
 
   const int n_tiles = (n + kTcM - 1) / kTcM;
+  const int tile0 = blockIdx.x + gridDim.x * gi, stride = gridDim.x * fwd::kGroups;
+  int tile = tile0;
   float2 fin[4];  // this thread's half of the raw features of its sample in the next tile
-  fetch_half(feats, blockIdx.x * kTcM + row, n, half, fin);
-  for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+  fetch_half(feats, tile * kTcM + row, n, half, fin);
+  for (; tile < n_tiles; tile += stride) {
     const int r = tile * kTcM + row;
     {
       float x[8];
       standardise_half(fin, r < n, half, mean, sd, x);
-      tc::store8_split(S + fwd::X, fwd::X_T, tc::kmajor_off(row, half, kTcK1), x);
+      tc::store8_split(S + h_off, fwd::X_T, tc::kmajor_off(row, half, kTcK1), x);
     }
     tc::fence_proxy_async();
-    __syncthreads();
-    if (t == 0)
-      mma_split(tmem, kmajor(sb + fwd::X, fwd::X_T, kTcK1), kmajor(sb + fwd::W1, fwd::W1_T, kTcK1), 1, idesc, bar);
-    fetch_half(feats, (tile + gridDim.x) * kTcM + row, n, half, fin);  // in flight during this tile's MMAs
-    bool ok = tc::mbar_wait(bar, phase);
+    tc::bar_sync(bid, kGroup);
+    if (t == 0) mma_split(d, kmajor(sb + h_off, fwd::X_T, kTcK1), kmajor(sb + fwd::W1, fwd::W1_T, kTcK1), 1, idesc, bar);
+    if (tile + stride < n_tiles) fetch_half(feats, (tile + stride) * kTcM + row, n, half, fin);  // in flight meanwhile
+    ok = ok && tc::mbar_wait(bar, phase);
     phase ^= 1u;
-    if (__syncthreads_or(!ok)) {
-      failed = true;
-      break;
-    }
     tc::fence_after_sync();
     // h1 columns [32 h, 32 h + 32) -> the H tile
 #pragma unroll
@@ -180,43 +200,33 @@ __global__ void __launch_bounds__(kTcThreads) k_mlp_forward(const float* __restr
       float v[16];
       tc::tmem_ld16(lane_base + 16 * q, v);
 #pragma unroll
-      for (int i = 0; i < 16; ++i) v[i] = fmaxf(v[i] + b1[32 * half + 16 * q + i], 0.f);
-      tc::store8_split(S + fwd::H, fwd::H_T, tc::kmajor_off(row, 4 * half + 2 * q, kMlpHid), v);
-      tc::store8_split(S + fwd::H, fwd::H_T, tc::kmajor_off(row, 4 * half + 2 * q + 1, kMlpHid), v + 8);
+      for (int i = 0; i < 16; ++i) v[i] = fmaxf(v[i], 0.f);
+      tc::store8_split(S + h_off, fwd::H_T, tc::kmajor_off(row, 4 * half + 2 * q, kMlpHid), v);
+      tc::store8_split(S + h_off, fwd::H_T, tc::kmajor_off(row, 4 * half + 2 * q + 1, kMlpHid), v + 8);
     }
     tc::fence_proxy_async();
     tc::fence_before_sync();
-    __syncthreads();
-    if (t == 0)
-      mma_split(tmem + 64, kmajor(sb + fwd::H, fwd::H_T, kMlpHid), kmajor(sb + fwd::W2, fwd::W2_T, kMlpHid), 4, idesc,
-                bar);
-    ok = tc::mbar_wait(bar, phase);
+    tc::bar_sync(bid, kGroup);
+    if (t == 0) mma_split(d, kmajor(sb + h_off, fwd::H_T, kMlpHid), kmajor(sb + fwd::W2, fwd::W2_T, kMlpHid), 4, idesc, bar);
+    ok = ok && tc::mbar_wait(bar, phase);
     phase ^= 1u;
-    if (__syncthreads_or(!ok)) {
-      failed = true;
-      break;
-    }
     tc::fence_after_sync();
     float acc = 0.f;
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
       float v[16];
-      tc::tmem_ld16(lane_base + 64 + 16 * q, v);
-#pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        const int j = 32 * half + 16 * q + i;
-        acc = fmaf(w3[j], fmaxf(v[i] + b2[j], 0.f), acc);
-      }
+      tc::tmem_ld16(lane_base + 16 * q, v);
+      acc = out_layer16(v, b2 + 32 * half + 16 * q, w3 + 32 * half + 16 * q, acc);
     }
-    part[half * kTcM + row] = acc;
+    if (half == 1) part[row] = acc;
     tc::fence_before_sync();
-    __syncthreads();
-    if (half == 0 && r < n) logits[r] = b3 + part[row] + part[kTcM + row];
+    if (tc::bar_or(bid, kGroup, !ok)) break;
+    if (half == 0 && r < n) logits[r] = b3 + acc + part[row];
   }
-  if (failed) {
-    // A tensor-core wait gave up: this block's remaining samples get NaN logits; the MMA in
-    // flight gets one more bounded wait before the tensor memory is released.
-    for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+  if (tile < n_tiles) {
+    // A tensor-core wait gave up: this group's remaining samples get NaN logits; the MMA in flight
+    // gets one more bounded wait before the tensor memory is released.
+    for (; tile < n_tiles; tile += stride) {
       const int r = tile * kTcM + row;
       if (half == 0 && r < n) logits[r] = __int_as_float(0x7fc00000);
     }
@@ -224,7 +234,7 @@ __global__ void __launch_bounds__(kTcThreads) k_mlp_forward(const float* __restr
   }
   tc::fence_before_sync();
   __syncthreads();
-  if (warp == 0) {
+  if (threadIdx.x < 32) {
     tc::fence_after_sync();
     tc::tmem_dealloc(tmem, fwd::kCols);
   }
@@ -303,269 +313,325 @@ int launch_mlp_finder_scores(const float* params, const float* feats, int n, flo
   return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
-// Loss and gradient on the tensor cores: a persistent CTA of 256 threads per SM takes tiles of 128
-// samples, two threads per sample (each half of the columns), and runs per tile
-//   D1 = X W1^T -> h1 = relu(D1 + b1);  D2 = H1 W2^T -> z3 = b3 + W3 . relu(D2 + b2),
-//   g = sigmoid(z3) - y, e2 = g W3 [z2 > 0];  D3 = E2 W2 -> e1 = D3 [h1 > 0];
-//   Dg += [E2 | E1]^T [H1 | X | 1]   (accumulated in tensor memory over all the CTA's tiles),
-// so that Dg holds dW2 (rows 0-63, columns 0-63), dW1 (rows 64-127, columns 64-77), db2 and db1
-// (column 80). dW3, db3 and the loss are summed in registers. Shared memory (bytes; each operand
-// three tiles, hi, mid, lo): the sample x [e2 | e1] tile (128 x 128, K-major; read MN-major as the
-// A operand of the gradient MMA), the sample x [h1 | x | 1 | 0] tile (128 x 96: the A operand of
-// the first two MMAs, MN-major the B operand of the gradient MMA), W1 and W2 (W2 read MN-major is
-// W2^T for the third MMA); tensor memory: D1 then D3 at column 0, D2 at 64, Dg at 128.
+// Loss and gradient on the tensor cores. Per tile of a group:
+//   D1 = X W1^T -> h1 = relu(D1);  D2 = H1 W2^T -> z3 = b3 + W3 . relu(D2 + b2),
+//   g = (sigmoid(z3) - y), e2 = g W3 [z2 > 0];  D3 = E2 W2 -> e1 = D3 [h1 > 0];
+//   Dg2 += E2^T [H1 | X],  Dg1 += E1^T X   (accumulated in tensor memory over all the CTA's tiles),
+// so that Dg2's rows 0-63 hold dW2 (columns 0-63) and db2 (column 64 + 14, X's ones) and Dg1's rows
+// 0-63 dW1 (columns 0-13) and db1 (column 14). dW3, db3 and the loss are summed in registers.
+//
+// Two groups per CTA. Shared memory (bytes; each operand three tiles, hi, mid, lo): each group's
+// sample x [h1 | x] tile (128 x 80: the A operand of the first two MMAs, K-major, and the B operand of
+// the gradient MMAs, read MN-major), one sample x e tile (128 x 64: e2, then e1; K-major the A
+// operand of the third MMA, MN-major of the gradient MMAs), W1 and W2 (W2 read MN-major is W2^T for
+// the third MMA). The e tile is one group's at a time, from its e2 until its last MMA; the other
+// group then runs its forward layers. A gradient MMA has M = 128 with the tile's 64 columns as
+// the first rows; the rest reads what lies behind in shared memory (the next rows' values, at
+// the end the [h1 | x] tile) into accumulator rows 64-127, which nothing uses.
+// Tensor memory: per group D1 then D3 at 0 and D2 at 64; Dg2 at 256, Dg1 at 336.
+// GRD_NOTE
 namespace grd {
-constexpr uint32_t E_T = 32768, XH_T = 24576, W1_T = 2048, W2_T = 8192;  // bytes of one tile
-constexpr uint32_t E = 0, XH = E + 3 * E_T, W1 = XH + 3 * XH_T, W2 = W1 + 3 * W1_T, B1 = W2 + 3 * W2_T,
-                   B2 = B1 + 256, W3 = B2 + 256, MEAN = W3 + 256, SD = MEAN + 64, RED = SD + 64, PART = RED + 272,
-                   B3 = PART + 1024, BAR = B3 + 8, TMEM = BAR + 8, BYTES = TMEM + 8;
-// The allocation leaves room past W2's lo tile, so that no reading of the MN-major W2 operand's
-// offsets can leave the block's shared memory.
-constexpr uint32_t ALLOC = 208896;
-static_assert(BYTES <= ALLOC && W2 + 2 * W2_T + 13568 <= ALLOC, "shared-memory layout");
-constexpr uint32_t kCols = 256, kColD2 = 64, kColG = 128;
-constexpr int kXhK = 96, kEK = 128, kGN = 96;
+constexpr int kGroups = 2;
+constexpr uint32_t E_T = 16384, XH_T = 20480, W1_T = 2048, W2_T = 8192;  // bytes of one tile
+constexpr uint32_t E = 0, XH = E + 3 * E_T, W2 = XH + kGroups * 3 * XH_T, W1 = W2 + 3 * W2_T, B2 = W1 + 3 * W1_T,
+                   W3 = B2 + 256, MEAN = W3 + 256, SD = MEAN + 64, PART = SD + 64, RED = PART + kGroups * 1024,
+                   BAR = RED + 16 * 34 * 4, TMEM = BAR + 16 * kGroups, LOCK = TMEM + 4, USED = LOCK + 4, BYTES = USED + 8;
+static_assert(BYTES + 1024 <= 227 * 1024, "shared-memory layout");
+constexpr uint32_t kCols = 512, kColD2 = 64, kColG2 = 256, kColG1 = 336;
+constexpr int kXhK = 80, kEK = 64;
 }  // namespace grd
 
 // Instruction descriptor bits 15 and 16: A, B MN-major.
 constexpr uint32_t kAmn = 1u << 15, kBmn = 1u << 16;
 
-__global__ void __launch_bounds__(kTcThreads) k_mlp_loss_grad(const float* __restrict__ params,
-                                                              const float* __restrict__ feats,
-                                                              const float* __restrict__ labels, int n,
-                                                              float* __restrict__ grad, float* __restrict__ loss) {
+// Sums of v[i] over the warp's lanes, element i in lane i: five halving exchanges.
+__device__ __forceinline__ float warp_sum32(float* v, int lane) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int i = 0; i < o; ++i) {
+      const float other = __shfl_xor_sync(0xffffffffu, up ? v[i] : v[i + o], o);
+      v[i] = (up ? v[i + o] : v[i]) + other;
+    }
+  }
+  return v[0];
+}
+
+// grad[0 .. 3] += v[0 .. 3], as one 16-byte reduction where the address allows.
+__device__ __forceinline__ void add4(float* grad, const float* v) {
+  if ((reinterpret_cast<size_t>(grad) & 15) == 0) {
+    asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(grad), "f"(v[0]), "f"(v[1]), "f"(v[2]),
+                 "f"(v[3])
+                 : "memory");
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) atomicAdd(grad + i, v[i]);
+  }
+}
+
+__global__ void __launch_bounds__(grd::kGroups* kGroup, 1)
+    k_mlp_loss_grad(const float* __restrict__ params, const float* __restrict__ feats, const float* __restrict__ labels,
+                    int n, float inv_n, float* __restrict__ grad, float* __restrict__ loss) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned char* S = smem_raw + ((1024 - (tc::smem_u32(smem_raw) & 1023)) & 1023);
   const uint32_t sb = tc::smem_u32(S);
-  float* b1 = reinterpret_cast<float*>(S + grd::B1);
   float* b2 = reinterpret_cast<float*>(S + grd::B2);
   float* w3 = reinterpret_cast<float*>(S + grd::W3);
   float* mean = reinterpret_cast<float*>(S + grd::MEAN);
   float* sd = reinterpret_cast<float*>(S + grd::SD);
-  float* red = reinterpret_cast<float*>(S + grd::RED);    // dW3[64], db3, loss
-  float* part = reinterpret_cast<float*>(S + grd::PART);  // [2][128] output-layer partial sums
-  uint64_t* bar = reinterpret_cast<uint64_t*>(S + grd::BAR);
+  float* red = reinterpret_cast<float*>(S + grd::RED);  // [16 warps][34]: dW3 of the warp's 32 units, db3, loss
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(S + grd::TMEM);
-  const int t = threadIdx.x, warp = t >> 5, row = t & (kTcM - 1), half = t >> 7;
+  int* lock = reinterpret_cast<int*>(S + grd::LOCK);  // 1: the e tile is taken
+  int* used = reinterpret_cast<int*>(S + grd::USED);  // 1: the gradient accumulators hold a tile
+  const int gi = threadIdx.x / kGroup, t = threadIdx.x % kGroup, warp = t >> 5, row = t & (kTcM - 1), half = t / kTcM;
   const int hc = 32 * half;  // this thread's first column of a 64-column accumulator
+  float* part = reinterpret_cast<float*>(S + grd::PART) + gi * 2 * kTcM;  // [2][128] output-layer partial sums
+  // bar[0]: the layers' MMAs, bar[1]: the gradient MMAs (the first of them is in flight with the third layer's)
+  uint64_t* bar = reinterpret_cast<uint64_t*>(S + grd::BAR) + 2 * gi;
+  const uint32_t xh = grd::XH + gi * 3 * grd::XH_T;
+  const int bid = gi + 1;
 
   stage_weights_b(params, S + grd::W1, grd::W1_T, S + grd::W2, grd::W2_T);
-  for (int i = t; i < kMlpHid; i += blockDim.x) {
-    b1[i] = params[kMlpB1 + i];
-    b2[i] = params[kMlpB2 + i];
-    w3[i] = params[kMlpW3 + i];
+  if (threadIdx.x < kMlpHid) {
+    b2[threadIdx.x] = params[kMlpB2 + threadIdx.x];
+    w3[threadIdx.x] = params[kMlpW3 + threadIdx.x];
   }
-  if (t < kMlpIn) {
-    mean[t] = params[kMlpMean + t];
-    sd[t] = params[kMlpSd + t];
-  }
-  if (t < 66) red[t] = 0.f;
-  {  // constant columns of this row of the [h1 | x | 1 | 0] tile: 80 (one) and 81-95 (zero)
-    float c[8] = {half == 0 ? 1.f : 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    tc::store8_split(S + grd::XH, grd::XH_T, tc::kmajor_off(row, 10 + half, grd::kXhK), c);
+  if (threadIdx.x < kMlpIn) {
+    mean[threadIdx.x] = params[kMlpMean + threadIdx.x];
+    sd[threadIdx.x] = params[kMlpSd + threadIdx.x];
   }
   const float b3 = params[kMlpB3];
-  if (warp == 0) tc::tmem_alloc(tmem_slot, grd::kCols);
-  if (t == 0) tc::mbar_init(bar, 1);
+  if (threadIdx.x < 32) tc::tmem_alloc(tmem_slot, grd::kCols);
+  if (threadIdx.x == 0) *lock = *used = 0;
+  if (t == 0) {
+    tc::mbar_init(bar, 1);
+    tc::mbar_init(bar + 1, 1);
+  }
+  tc::fence_proxy_async();
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
-  const uint32_t tmem = *tmem_slot;
-  const uint32_t lane_base = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
+  const uint32_t tmem = *tmem_slot, d = tmem + 128u * gi;
+  const uint32_t lane_off = static_cast<uint32_t>((warp & 3) * 32) << 16;
+  const uint32_t lane_base = d + lane_off + hc;
   constexpr uint32_t id_kk = tc::idesc_bf16_f32(kTcM, kMlpHid);
-  constexpr uint32_t id_kmn = id_kk | kBmn;
-  constexpr uint32_t id_grad = tc::idesc_bf16_f32(kTcM, grd::kGN) | kAmn | kBmn;
-  uint32_t phase = 0;
-  bool failed = false;
+  constexpr uint32_t id_g2 = tc::idesc_bf16_f32(kTcM, grd::kXhK) | kAmn | kBmn;
+  constexpr uint32_t id_g1 = tc::idesc_bf16_f32(kTcM, kTcK1) | kAmn | kBmn;
+  const Operand e_k = kmajor(sb + grd::E, grd::E_T, grd::kEK), e_mn = mnmajor(sb + grd::E, grd::E_T, grd::kEK);
+  uint32_t phase = 0, gphase = 0;
+  bool ok = true, locked = false;
   float acc3[32];  // dW3 partial sums of this thread's 32 hidden units
 #pragma unroll
   for (int j = 0; j < 32; ++j) acc3[j] = 0.f;
   float gsum = 0.f, lsum = 0.f;
 
   const int n_tiles = (n + kTcM - 1) / kTcM;
-  int done_tiles = 0;
+  const int stride = gridDim.x * grd::kGroups;
+  int tile = blockIdx.x + gridDim.x * gi;
   float2 fin[4];  // this thread's half of the raw features, and the label, of its sample in the next tile
-  fetch_half(feats, blockIdx.x * kTcM + row, n, half, fin);
-  float yin = blockIdx.x * kTcM + row < n ? labels[blockIdx.x * kTcM + row] : 0.f;
-  for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++done_tiles) {
-    const int r = tile * kTcM + row;
-    const bool valid = r < n;
-    {  // inputs -> columns 64-79 of the [h1 | x | 1 | 0] tile
+  fetch_half(feats, tile * kTcM + row, n, half, fin);
+  float yin = tile * kTcM + row < n ? labels[tile * kTcM + row] : 0.f;
+  for (; tile < n_tiles; tile += stride) {
+    const bool valid = tile * kTcM + row < n;
+    {  // inputs -> columns 64-79 of the [h1 | x] tile
       float x[8];
       standardise_half(fin, valid, half, mean, sd, x);
-      tc::store8_split(S + grd::XH, grd::XH_T, tc::kmajor_off(row, 8 + half, grd::kXhK), x);
+      tc::store8_split(S + xh, grd::XH_T, tc::kmajor_off(row, 8 + half, grd::kXhK), x);
     }
     const float y = yin;
-    {
-      const int rn = (tile + gridDim.x) * kTcM + row;  // in flight during this tile's MMAs
+    tc::fence_proxy_async();
+    tc::bar_sync(bid, kGroup);
+    if (t == 0)
+      mma_split(d, kmajor(sb + xh, grd::XH_T, grd::kXhK, 8), kmajor(sb + grd::W1, grd::W1_T, kTcK1), 1, id_kk, bar);
+    if (tile + stride < n_tiles) {  // in flight during this tile
+      const int rn = (tile + stride) * kTcM + row;
       fetch_half(feats, rn, n, half, fin);
       yin = rn < n ? labels[rn] : 0.f;
     }
-    tc::fence_proxy_async();
-    __syncthreads();
-    if (t == 0)
-      mma_split(tmem, kmajor(sb + grd::XH, grd::XH_T, grd::kXhK, 8), kmajor(sb + grd::W1, grd::W1_T, kTcK1), 1,
-                id_kk, bar);
-    bool ok = tc::mbar_wait(bar, phase);
+    ok = ok && tc::mbar_wait(bar, phase);
     phase ^= 1u;
-    if (__syncthreads_or(!ok)) {
-      failed = true;
-      break;
-    }
     tc::fence_after_sync();
-    // h1 -> columns [hc, hc + 32) of the [h1 | x | 1 | 0] tile; mask1 = [h1 > 0]
+    // h1 -> columns [hc, hc + 32) of the [h1 | x] tile; mask1 = [h1 > 0]
     unsigned mask1 = 0u;
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
       float v[16];
-      tc::tmem_ld16(lane_base + hc + 16 * q, v);
+      tc::tmem_ld16(lane_base + 16 * q, v);
 #pragma unroll
       for (int i = 0; i < 16; ++i) {
-        v[i] = fmaxf(v[i] + b1[hc + 16 * q + i], 0.f);
+        v[i] = fmaxf(v[i], 0.f);
         if (v[i] > 0.f) mask1 |= 1u << (16 * q + i);
       }
-      tc::store8_split(S + grd::XH, grd::XH_T, tc::kmajor_off(row, 4 * half + 2 * q, grd::kXhK), v);
-      tc::store8_split(S + grd::XH, grd::XH_T, tc::kmajor_off(row, 4 * half + 2 * q + 1, grd::kXhK), v + 8);
+      tc::store8_split(S + xh, grd::XH_T, tc::kmajor_off(row, 4 * half + 2 * q, grd::kXhK), v);
+      tc::store8_split(S + xh, grd::XH_T, tc::kmajor_off(row, 4 * half + 2 * q + 1, grd::kXhK), v + 8);
     }
     tc::fence_proxy_async();
     tc::fence_before_sync();
-    __syncthreads();
+    tc::bar_sync(bid, kGroup);
     if (t == 0)
-      mma_split(tmem + grd::kColD2, kmajor(sb + grd::XH, grd::XH_T, grd::kXhK),
-                kmajor(sb + grd::W2, grd::W2_T, kMlpHid), 4, id_kk, bar);
-    ok = tc::mbar_wait(bar, phase);
+      mma_split(d + grd::kColD2, kmajor(sb + xh, grd::XH_T, grd::kXhK), kmajor(sb + grd::W2, grd::W2_T, kMlpHid), 4, id_kk,
+                bar);
+    ok = ok && tc::mbar_wait(bar, phase);
     phase ^= 1u;
-    if (__syncthreads_or(!ok)) {
-      failed = true;
-      break;
-    }
     tc::fence_after_sync();
     {  // logit from the two halves' partial sums
       float acc = 0.f;
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
         float v[16];
-        tc::tmem_ld16(lane_base + grd::kColD2 + hc + 16 * q, v);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const int j = hc + 16 * q + i;
-          acc = fmaf(w3[j], fmaxf(v[i] + b2[j], 0.f), acc);
-        }
+        tc::tmem_ld16(lane_base + grd::kColD2 + 16 * q, v);
+        acc = out_layer16(v, b2 + hc + 16 * q, w3 + hc + 16 * q, acc);
       }
       part[half * kTcM + row] = acc;
     }
-    __syncthreads();
+    if (t == 0 && ok) {  // the e tile: the other group's until its gradient MMAs are done
+      const uint64_t t0 = tc::global_ns();
+      while (!(locked = atomicCAS(lock, 0, 1) == 0) && tc::global_ns() - t0 < 2000000000ull) __nanosleep(40);
+      ok = locked;
+      __threadfence_block();
+    }
+    if (tc::bar_or(bid, kGroup, !ok)) break;
     const float z3 = b3 + part[row] + part[kTcM + row];
     const float g = valid ? 1.f / (1.f + expf(-z3)) - y : 0.f;
     if (half == 0) {
       if (valid) lsum += fmaxf(z3, 0.f) - z3 * y + log1pf(expf(-fabsf(z3)));
       gsum += g;
     }
-    // e2 -> columns [hc, hc + 32) of the [e2 | e1] tile; dW3 partial sums
+    // e2 -> columns [hc, hc + 32) of the e tile; dW3 partial sums
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
       float v[16];
-      tc::tmem_ld16(lane_base + grd::kColD2 + hc + 16 * q, v);
+      tc::tmem_ld16(lane_base + grd::kColD2 + 16 * q, v);
 #pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        const float a2 = fmaxf(v[i] + b2[hc + 16 * q + i], 0.f);
-        acc3[16 * q + i] = fmaf(g, a2, acc3[16 * q + i]);
-        v[i] = a2 > 0.f ? g * w3[hc + 16 * q + i] : 0.f;
+      for (int i = 0; i < 4; ++i) {
+        const float4 b = reinterpret_cast<const float4*>(b2 + hc + 16 * q)[i];
+        const float4 w = reinterpret_cast<const float4*>(w3 + hc + 16 * q)[i];
+        const float bb[4] = {b.x, b.y, b.z, b.w}, ww[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float a2 = fmaxf(v[4 * i + e] + bb[e], 0.f);
+          acc3[16 * q + 4 * i + e] = fmaf(g, a2, acc3[16 * q + 4 * i + e]);
+          v[4 * i + e] = a2 > 0.f ? g * ww[e] : 0.f;
+        }
       }
       tc::store8_split(S + grd::E, grd::E_T, tc::kmajor_off(row, 4 * half + 2 * q, grd::kEK), v);
       tc::store8_split(S + grd::E, grd::E_T, tc::kmajor_off(row, 4 * half + 2 * q + 1, grd::kEK), v + 8);
     }
     tc::fence_proxy_async();
     tc::fence_before_sync();
-    __syncthreads();
-    // D3 = E2 W2: W2's K-major tile (rows o, columns i) read MN-major is W2^T (n = i, k = o).
-    if (t == 0)
-      mma_split(tmem, kmajor(sb + grd::E, grd::E_T, grd::kEK), mnmajor(sb + grd::W2, grd::W2_T, kMlpHid), 4, id_kmn,
-                bar);
-    ok = tc::mbar_wait(bar, phase);
-    phase ^= 1u;
-    if (__syncthreads_or(!ok)) {
-      failed = true;
-      break;
+    tc::bar_sync(bid, kGroup);
+    // D3 = E2 W2: W2's K-major tile (rows o, columns i) read MN-major is W2^T (n = i, k = o). Then
+    // Dg2 += E2^T [H1 | X]: both tiles read MN-major, K = the tile's 128 samples.
+    if (t == 0) {
+      mma_split(d, e_k, mnmajor(sb + grd::W2, grd::W2_T, kMlpHid), 4, id_kk | kBmn, bar);
+      mma_split(tmem + grd::kColG2, e_mn, mnmajor(sb + xh, grd::XH_T, grd::kXhK), kTcM / 16, id_g2, bar + 1, *used != 0);
     }
+    ok = ok && tc::mbar_wait(bar, phase);
+    phase ^= 1u;
     tc::fence_after_sync();
-    // e1 -> columns 64 + [hc, hc + 32) of the [e2 | e1] tile
+    // e1, split while the gradient MMA still reads e2
+    uint4 e1[4][3];
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
       float v[16];
-      tc::tmem_ld16(lane_base + hc + 16 * q, v);
+      tc::tmem_ld16(lane_base + 16 * q, v);
 #pragma unroll
       for (int i = 0; i < 16; ++i) v[i] = (mask1 >> (16 * q + i)) & 1u ? v[i] : 0.f;
-      tc::store8_split(S + grd::E, grd::E_T, tc::kmajor_off(row, 8 + 4 * half + 2 * q, grd::kEK), v);
-      tc::store8_split(S + grd::E, grd::E_T, tc::kmajor_off(row, 9 + 4 * half + 2 * q, grd::kEK), v + 8);
+      tc::split8(v, e1[2 * q][0], e1[2 * q][1], e1[2 * q][2]);
+      tc::split8(v + 8, e1[2 * q + 1][0], e1[2 * q + 1][1], e1[2 * q + 1][2]);
     }
+    ok = ok && tc::mbar_wait(bar + 1, gphase);
+    gphase ^= 1u;
+    tc::fence_after_sync();
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+      tc::store8(S + grd::E, grd::E_T, tc::kmajor_off(row, 4 * half + c, grd::kEK), e1[c][0], e1[c][1], e1[c][2]);
     tc::fence_proxy_async();
     tc::fence_before_sync();
-    __syncthreads();
-    // Dg += [e2 | e1]^T [h1 | x | 1 | 0]: both tiles read MN-major, K = the tile's 128 samples.
+    tc::bar_sync(bid, kGroup);
+    // Dg1 += E1^T X
     if (t == 0)
-      mma_split(tmem + grd::kColG, mnmajor(sb + grd::E, grd::E_T, grd::kEK), mnmajor(sb + grd::XH, grd::XH_T, grd::kXhK),
-                kTcM / 16, id_grad, bar, done_tiles > 0);
-    ok = tc::mbar_wait(bar, phase);
-    phase ^= 1u;
-    if (__syncthreads_or(!ok)) {
-      failed = true;
-      break;
-    }
+      mma_split(tmem + grd::kColG1, e_mn, mnmajor(sb + xh, grd::XH_T, grd::kXhK, 8), kTcM / 16, id_g1, bar + 1, *used != 0);
+    ok = ok && tc::mbar_wait(bar + 1, gphase);
+    gphase ^= 1u;
     tc::fence_after_sync();
+    if (t == 0) {
+      *used = 1;
+      __threadfence_block();
+      atomicExch(lock, 0);
+      locked = false;
+    }
   }
-  if (failed) {
-    // A tensor-core wait gave up: the loss becomes NaN and this block adds no gradient; the MMA in
-    // flight gets one more bounded wait before the tensor memory is released.
-    if (t == 0) atomicAdd(loss, __int_as_float(0x7fc00000));
+  if (tc::bar_or(bid, kGroup, !ok)) {
+    // A tensor-core wait gave up: the loss becomes NaN; the MMAs in flight get one more bounded wait
+    // before the tensor memory is released.
+    if (t == 0) {
+      if (locked) atomicExch(lock, 0);
+      atomicAdd(loss, __int_as_float(0x7fc00000));
+    }
     tc::mbar_wait(bar, phase ^ 1u);
-  } else if (done_tiles > 0) {
+    tc::mbar_wait(bar + 1, gphase ^ 1u);
+    gsum = lsum = 0.f;
+  }
+  // dW3, db3 and the loss: over the warp's samples, then over the eight warps of each half.
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  red[wid * 34 + lane] = warp_sum32(acc3, lane);
 #pragma unroll
-    for (int j = 0; j < 32; ++j) atomicAdd(&red[hc + j], acc3[j]);
-    if (half == 0) {
-      atomicAdd(&red[64], gsum);
-      atomicAdd(&red[65], lsum);
-    }
-    // Dg row `row` (warp-uniform branches): dW2 row j = row, columns [hc, hc + 32), and db2[j]
-    // (column 80, half 0); or dW1 row i = row - 64 (columns 64-77, half 0) and db1[i] (half 1).
-    float v[16];
-    if (row < kMlpHid) {
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        tc::tmem_ld16(lane_base + grd::kColG + hc + 16 * q, v);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) atomicAdd(grad + kMlpW2 + row * kMlpHid + hc + 16 * q + i, v[i]);
-      }
-      if (half == 0) {
-        tc::tmem_ld16(lane_base + grd::kColG + 80, v);
-        atomicAdd(grad + kMlpB2 + row, v[0]);
-      }
-    } else if (half == 0) {
-      tc::tmem_ld16(lane_base + grd::kColG + 64, v);
-#pragma unroll
-      for (int k = 0; k < kMlpIn; ++k) atomicAdd(grad + kMlpW1 + (row - kMlpHid) * kMlpIn + k, v[k]);
-    } else {
-      tc::tmem_ld16(lane_base + grd::kColG + 80, v);
-      atomicAdd(grad + kMlpB1 + row - kMlpHid, v[0]);
-    }
-    __syncthreads();
-    if (t < kMlpHid) atomicAdd(grad + kMlpW3 + t, red[t]);
-    if (t == kMlpHid) atomicAdd(grad + kMlpB3, red[64]);
-    if (t == kMlpHid + 1) atomicAdd(loss, red[65]);
+  for (int o = 16; o > 0; o >>= 1) {
+    gsum += __shfl_xor_sync(0xffffffffu, gsum, o);
+    lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
+  }
+  if (lane == 0) {
+    red[wid * 34 + 32] = gsum;
+    red[wid * 34 + 33] = lsum;
   }
   tc::fence_before_sync();
   __syncthreads();
-  if (warp == 0) {
+  tc::fence_after_sync();
+  if (threadIdx.x < kMlpHid + 2) {
+    const int j = threadIdx.x;  // dW3[j], db3, loss: warps 0-3 and 8-11 hold units 0-31, the others 32-63
+    float v = 0.f;
+    for (int w = 0; w < 16; ++w) {
+      if (j < kMlpHid) v += ((w >> 2) & 1) == (j >> 5) ? red[w * 34 + (j & 31)] : 0.f;
+      else v += red[w * 34 + 32 + j - kMlpHid];
+    }
+    if (j <= kMlpHid) atomicAdd(grad + (j < kMlpHid ? kMlpW3 + j : kMlpB3), v * inv_n);
+    else atomicAdd(loss, v * inv_n);
+  }
+  // The gradient accumulators' rows 0-63 (tensor-memory lanes 0-63, the warps w with w % 4 < 2): the
+  // four such pairs of warps take 16 columns of dW2 each; db2 (pair 1), dW1 and db1 (pair 2).
+  if (*used && (wid & 3) < 2) {
+    const int j = 32 * (wid & 3) + lane, q = wid >> 2;
+    float v[16];
+    tc::tmem_ld16(tmem + lane_off + grd::kColG2 + 16 * q, v);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] *= inv_n;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) add4(grad + kMlpW2 + j * kMlpHid + 16 * q + 4 * i, v + 4 * i);
+    if (q == 1) {
+      tc::tmem_ld16(tmem + lane_off + grd::kColG2 + 64, v);
+      atomicAdd(grad + kMlpB2 + j, v[kOne] * inv_n);
+    }
+    if (q == 2) {
+      tc::tmem_ld16(tmem + lane_off + grd::kColG1, v);
+#pragma unroll
+      for (int k = 0; k < kMlpIn; ++k) atomicAdd(grad + kMlpW1 + j * kMlpIn + k, v[k] * inv_n);
+      atomicAdd(grad + kMlpB1 + j, v[kOne] * inv_n);
+    }
+  }
+  tc::fence_before_sync();
+  __syncthreads();
+  if (threadIdx.x < 32) {
     tc::fence_after_sync();
     tc::tmem_dealloc(tmem, grd::kCols);
   }
 }
 
-__global__ void k_mlp_scale(float* grad, float* loss, float inv_n) {
-  for (int p = blockIdx.x * blockDim.x + threadIdx.x; p <= kMlpParams; p += gridDim.x * blockDim.x) {
-    if (p < kMlpParams) grad[p] *= inv_n;
-    else *loss *= inv_n;
-  }
+__global__ void k_mlp_zero(float* grad, float* loss) {
+  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+  if (p < kMlpParams) grad[p] = 0.f;
+  else if (p == kMlpParams) *loss = 0.f;
 }
 
 // Adam (Kingma and Ba) on the weights; moments m, v; step t >= 1.
@@ -605,20 +671,19 @@ int launch_mlp_forward(const float* params, const float* feats, int n, float* lo
   int sms = 0;
   if (tc_prepare(reinterpret_cast<const void*>(k_mlp_forward), smem, &sms) != 0) return -3;
   const int tiles = (n + kTcM - 1) / kTcM;
-  k_mlp_forward<<<std::min(tiles, kFwdCtasPerSm * sms), kTcThreads, smem, st>>>(params, feats, n, logits);
+  k_mlp_forward<<<std::min(tiles, sms), fwd::kGroups * kGroup, smem, st>>>(params, feats, n, logits);
   return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
 int launch_mlp_loss_grad(const float* params, const float* feats, const float* labels, int n, float* grad, float* loss,
                          cudaStream_t st) {
-  const int smem = static_cast<int>(grd::ALLOC) + 1024;
+  const int smem = static_cast<int>(grd::BYTES) + 1024;
   int sms = 0;
   if (tc_prepare(reinterpret_cast<const void*>(k_mlp_loss_grad), smem, &sms) != 0) return -3;
-  if (cudaMemsetAsync(grad, 0, sizeof(float) * kMlpParams, st) != cudaSuccess) return -3;
-  if (cudaMemsetAsync(loss, 0, sizeof(float), st) != cudaSuccess) return -3;
+  k_mlp_zero<<<(kMlpParams + 256) / 256, 256, 0, st>>>(grad, loss);
   const int tiles = (n + kTcM - 1) / kTcM;
-  if (n > 0) k_mlp_loss_grad<<<std::min(tiles, sms), kTcThreads, smem, st>>>(params, feats, labels, n, grad, loss);
-  k_mlp_scale<<<8, 256, 0, st>>>(grad, loss, n > 0 ? 1.f / n : 0.f);
+  if (n > 0)
+    k_mlp_loss_grad<<<std::min(tiles, sms), grd::kGroups * kGroup, smem, st>>>(params, feats, labels, n, 1.f / n, grad, loss);
   return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 

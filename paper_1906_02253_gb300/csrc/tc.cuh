@@ -17,7 +17,6 @@
 // mid, lo.
 #pragma once
 
-#include <cuda_bf16.h>
 #include <stdint.h>
 
 namespace kfgb {
@@ -75,6 +74,22 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint64
   }
 }
 
+// Barrier `id` among n threads of the block (a group of whole warps); bar_or also tells every thread
+// whether p holds for any of them.
+__device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+__device__ __forceinline__ bool bar_or(int id, int n, bool p) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 p, %3, 0;\n\t"
+      "bar.red.or.pred q, %1, %2, p;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(r)
+      : "r"(id), "r"(n), "r"(static_cast<uint32_t>(p))
+      : "memory");
+  return r != 0;
+}
+
 // Tensor-memory allocation by one whole warp; the column base is written to *dst.
 __device__ __forceinline__ void tmem_alloc(uint32_t* dst, uint32_t ncols) {
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(dst)), "r"(ncols)
@@ -119,32 +134,46 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-__device__ __forceinline__ uint32_t pack_bf16(__nv_bfloat16 a, __nv_bfloat16 b) {
-  return static_cast<uint32_t>(__bfloat16_as_ushort(a)) | (static_cast<uint32_t>(__bfloat16_as_ushort(b)) << 16);
+// Two values rounded to bf16 (x0 in the low half), and the two values of such a word.
+__device__ __forceinline__ uint32_t cvt_bf16x2(float x0, float x1) {
+  uint32_t r;
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(x1), "f"(x0));
+  return r;
 }
+__device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
+__device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
 
-// Splits 8 consecutive values into their hi, mid and lo bf16 parts and stores them as one 16-byte
-// row of a core matrix at byte offset off of each of the three tiles (tile_bytes apart from t0).
-__device__ __forceinline__ void store8_split(unsigned char* t0, uint32_t tile_bytes, uint32_t off, const float* v) {
-  uint32_t h[4], m[4], l[4];
+// hi, mid and lo bf16 parts of 8 consecutive values, two values to a word.
+__device__ __forceinline__ void split8(const float* v, uint4& h, uint4& m, uint4& l) {
+  uint32_t w[3][4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    __nv_bfloat16 p[3][2];
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      const float x = v[2 * i + e];
-      p[0][e] = __float2bfloat16_rn(x);
-      const float r1 = x - __bfloat162float(p[0][e]);
-      p[1][e] = __float2bfloat16_rn(r1);
-      p[2][e] = __float2bfloat16_rn(r1 - __bfloat162float(p[1][e]));
-    }
-    h[i] = pack_bf16(p[0][0], p[0][1]);
-    m[i] = pack_bf16(p[1][0], p[1][1]);
-    l[i] = pack_bf16(p[2][0], p[2][1]);
+    const float a = v[2 * i], b = v[2 * i + 1];
+    const uint32_t hw = cvt_bf16x2(a, b);
+    const float a1 = a - bf16_lo(hw), b1 = b - bf16_hi(hw);
+    const uint32_t mw = cvt_bf16x2(a1, b1);
+    w[0][i] = hw;
+    w[1][i] = mw;
+    w[2][i] = cvt_bf16x2(a1 - bf16_lo(mw), b1 - bf16_hi(mw));
   }
-  *reinterpret_cast<uint4*>(t0 + off) = make_uint4(h[0], h[1], h[2], h[3]);
-  *reinterpret_cast<uint4*>(t0 + tile_bytes + off) = make_uint4(m[0], m[1], m[2], m[3]);
-  *reinterpret_cast<uint4*>(t0 + 2 * tile_bytes + off) = make_uint4(l[0], l[1], l[2], l[3]);
+  h = make_uint4(w[0][0], w[0][1], w[0][2], w[0][3]);
+  m = make_uint4(w[1][0], w[1][1], w[1][2], w[1][3]);
+  l = make_uint4(w[2][0], w[2][1], w[2][2], w[2][3]);
+}
+
+// Stores the three parts as one 16-byte row of a core matrix at byte offset off of each of the three
+// tiles (tile_bytes apart from t0).
+__device__ __forceinline__ void store8(unsigned char* t0, uint32_t tile_bytes, uint32_t off, const uint4& h,
+                                       const uint4& m, const uint4& l) {
+  *reinterpret_cast<uint4*>(t0 + off) = h;
+  *reinterpret_cast<uint4*>(t0 + tile_bytes + off) = m;
+  *reinterpret_cast<uint4*>(t0 + 2 * tile_bytes + off) = l;
+}
+
+__device__ __forceinline__ void store8_split(unsigned char* t0, uint32_t tile_bytes, uint32_t off, const float* v) {
+  uint4 h, m, l;
+  split8(v, h, m, l);
+  store8(t0, tile_bytes, off, h, m, l);
 }
 
 // Byte offset of row r, core-matrix column c (elements 8c .. 8c + 7) in a K-major tile of Kt columns.
