@@ -25,19 +25,51 @@ constexpr int kTcK1 = 16;   // inputs padded to one MMA K step
 constexpr int kOne = kMlpIn;  // the input that is one
 constexpr int kGroup = 2 * kTcM;
 
-// Inference: per tile, standardised inputs -> X tile (128 x 16); D = X W1^T in tensor memory; h1 =
-// relu(D) -> H tile (128 x 64, over the X tile, which the finished MMA no longer needs); D = H W2^T;
-// logit = b3 + sum_j W3[j] relu(D[j] + b2[j]) on the CUDA cores. Four groups per CTA (1024 threads
-// at 64 registers; shared memory for four H tiles and one set of weights): on 1,000,003 rows
-// FWD_NOTE
+// Hidden activations as the A operand of the next layer: the parts go to tensor memory, 16 columns
+// of a thread's 32 at a time. With A in shared memory every MMA of K = 16 read 4 KB for A and 2 KB
+// for B there, 48 cycles of its bandwidth for 32 cycles of tensor work. The columns may be those of
+// the accumulator that the activations came from: a thread's hi and mid parts lie in the 32 columns
+// that it reads itself (half h: 32 h + 0-15 hi, 32 h + 16-31 mid; lo at 64 + 16 h).
+struct Parts {
+  uint4 h[4], m[4], l[4];  // 8 columns each
+};
+__device__ __forceinline__ void split16(const float* v, int q, Parts& p) {
+  tc::split8(v, p.h[2 * q], p.m[2 * q], p.l[2 * q]);
+  tc::split8(v + 8, p.h[2 * q + 1], p.m[2 * q + 1], p.l[2 * q + 1]);
+}
+template <bool LO>
+__device__ __forceinline__ void parts_to_tmem(uint32_t region, int half, int q, const Parts& p) {
+  tc::tmem_st8(region + 32 * half + 8 * q, p.h[2 * q], p.h[2 * q + 1]);
+  tc::tmem_st8(region + 32 * half + 16 + 8 * q, p.m[2 * q], p.m[2 * q + 1]);
+  if (LO) tc::tmem_st8(region + 64 + 16 * half + 8 * q, p.l[2 * q], p.l[2 * q + 1]);
+}
+// This thread's parts of columns [32 half, 32 half + 32) into a K-major tile of KT columns, the hi,
+// mid and lo parts starting at its column blocks H, M and L.
+template <int KT, int H, int M, int L>
+__device__ __forceinline__ void parts_to_smem(unsigned char* t0, int row, int half, const Parts& p) {
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    *reinterpret_cast<uint4*>(t0 + tc::kmajor_off(row, H + 4 * half + c, KT)) = p.h[c];
+    *reinterpret_cast<uint4*>(t0 + tc::kmajor_off(row, M + 4 * half + c, KT)) = p.m[c];
+    *reinterpret_cast<uint4*>(t0 + tc::kmajor_off(row, L + 4 * half + c, KT)) = p.l[c];
+  }
+}
+
+// Inference: per tile, standardised inputs -> X tile (128 x 16); D1 = X W1^T in tensor memory; h1 =
+// relu(D1) -> the next A operand (in D1's columns; its lo part over the X tile, which the finished
+// MMA no longer needs); D2 = H W2^T; logit = b3 + sum_j W3[j] relu(D2[j] + b2[j]) on the CUDA cores.
+// Four groups per CTA (1024 threads at 64 registers, all 512 tensor-memory columns). 1,000,003 rows take
+// 55 us (183 TFLOP/s of the network's flops, six times that on the tensor cores: 58% of the measured
+// bf16 rate), where one chain per CTA, two CTAs per SM, took 115 us; the bound is the CUDA cores'
+// issue rate (splits, ReLU, output layer), then the tensor pipe.
 namespace fwd {
 constexpr int kGroups = 4;
 constexpr uint32_t W1_T = 2048, W2_T = 8192, H_T = 16384, X_T = 4096;  // bytes of one tile
-constexpr uint32_t W1 = 0, W2 = W1 + 3 * W1_T, H = W2 + 3 * W2_T, B2 = H + kGroups * 3 * H_T, W3 = B2 + 256,
-                   MEAN = W3 + 256, SD = MEAN + 64, PART = SD + 64, BAR = PART + kGroups * 512, TMEM = BAR + 8 * kGroups,
+constexpr uint32_t W1 = 0, W2 = W1 + 3 * W1_T, H = W2 + 3 * W2_T, B2 = H + kGroups * H_T, W3 = B2 + 256,
+                   MEAN = W3 + 256, SD = MEAN + 64, RS = SD + 64, PART = RS + 64, BAR = PART + kGroups * 512, TMEM = BAR + 8 * kGroups,
                    BYTES = TMEM + 8;
-constexpr uint32_t kCols = 64 * kGroups;
-static_assert(BYTES + 1024 <= 227 * 1024 && 3 * X_T <= 3 * H_T, "shared-memory layout");
+constexpr uint32_t kCols = 128 * kGroups;
+static_assert(BYTES + 1024 <= 227 * 1024 && 3 * X_T <= H_T, "shared-memory layout");
 }  // namespace fwd
 
 // Loads W1 (64 x 16: 14 inputs, b1, zero) and W2 (64 x 64) as the MMAs' B operands in the K-major
@@ -74,64 +106,126 @@ __device__ __forceinline__ void fetch_half(const float* __restrict__ feats, int 
   }
 }
 
-// Standardised inputs [8 h, 8 h + 8) into x[8] (zero past n), the one and the zero.
-__device__ __forceinline__ void standardise_half(const float2* f, bool valid, int half, const float* mean,
-                                                 const float* sd, float* x) {
+// Normaliser in shared memory, 16 entries each: mean, sd and 1 / sd; the inputs past the 14, fetched as
+// zeros, become the one and the zero. Tells whether each sd is within [2^-100, 2^100], where the
+// reciprocal form below gives the quotient.
+__device__ __forceinline__ bool stage_normaliser(const float* __restrict__ params, float* mean, float* sd, float* rs) {
+  const int t = threadIdx.x;
+  bool in_range = true;
+  if (t < kTcK1) {
+    const float s = t < kMlpIn ? params[kMlpSd + t] : 1.f;
+    mean[t] = t < kMlpIn ? params[kMlpMean + t] : t == kOne ? -1.f : 0.f;
+    sd[t] = s;
+    rs[t] = 1.f / s;
+    in_range = fabsf(s) >= 7.8886091e-31f && fabsf(s) <= 1.2676506e30f;
+  }
+  return in_range;
+}
+
+// Standardised inputs [8 h, 8 h + 8), split for their tile. The quotient is a / sd from its
+// reciprocal with one correction by the remainder (divisions were a seventh of the forward pass's
+// instructions). Rows past n hold some finite value here: nothing of theirs is written or summed.
+__device__ __forceinline__ void standardise_half(const float2* f, int half, const float* mean, const float* sd,
+                                                 const float* rs, bool by_reciprocal, uint4 (&x)[3]) {
+  float v[8];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const int k = 8 * half + 2 * i;
-    x[2 * i] = (valid && k < kMlpIn) ? (f[i].x - mean[k]) / sd[k] : 0.f;
-    x[2 * i + 1] = (valid && k + 1 < kMlpIn) ? (f[i].y - mean[k + 1]) / sd[k + 1] : 0.f;
+    const float2 m = *reinterpret_cast<const float2*>(mean + k), s = *reinterpret_cast<const float2*>(sd + k);
+    const float2 r = *reinterpret_cast<const float2*>(rs + k);
+    const uint64_t a = tc::sub2(tc::pack2(f[i].x, f[i].y), tc::pack2(m.x, m.y)), rr = tc::pack2(r.x, r.y);
+    if (by_reciprocal) {
+      const uint64_t q = tc::mul2(a, rr);
+      tc::unpack2(tc::fma2(tc::fma2(q, tc::pack2(-s.x, -s.y), a), rr, q), v[2 * i], v[2 * i + 1]);
+    } else {
+      float a0, a1;
+      tc::unpack2(a, a0, a1);
+      v[2 * i] = a0 / s.x;
+      v[2 * i + 1] = a1 / s.y;
+    }
   }
-  if (half == 1) x[kOne - 8] = 1.f;
+  tc::split8(v, x[0], x[1], x[2]);
 }
 
-// This thread's 16 columns [c, c + 16) of sum_j w3[j] relu(v[j] + b2[j]) onto acc (columns 16-byte
-// aligned in shared memory).
-__device__ __forceinline__ float out_layer16(const float* v, const float* b2, const float* w3, float acc) {
+// relu(v + b2) of this thread's 16 columns [c, c + 16) (16-byte aligned in shared memory), in place.
+__device__ __forceinline__ void relu16(float* v, const float* b2) {
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const float4 b = reinterpret_cast<const float4*>(b2)[i], w = reinterpret_cast<const float4*>(w3)[i];
-    acc = fmaf(w.x, fmaxf(v[4 * i] + b.x, 0.f), acc);
-    acc = fmaf(w.y, fmaxf(v[4 * i + 1] + b.y, 0.f), acc);
-    acc = fmaf(w.z, fmaxf(v[4 * i + 2] + b.z, 0.f), acc);
-    acc = fmaf(w.w, fmaxf(v[4 * i + 3] + b.w, 0.f), acc);
+    const float4 b = reinterpret_cast<const float4*>(b2)[i];
+    tc::unpack2(tc::add2(tc::pack2(v[4 * i], v[4 * i + 1]), tc::pack2(b.x, b.y)), v[4 * i], v[4 * i + 1]);
+    tc::unpack2(tc::add2(tc::pack2(v[4 * i + 2], v[4 * i + 3]), tc::pack2(b.z, b.w)), v[4 * i + 2], v[4 * i + 3]);
+  }
+#pragma unroll
+  for (int i = 0; i < 16; ++i) v[i] = fmaxf(v[i], 0.f);
+}
+
+// acc += the even and odd terms of sum_j w3[j] v[j] over 16 columns.
+__device__ __forceinline__ uint64_t dot16(const float* v, const float* w3, uint64_t acc) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const float4 w = reinterpret_cast<const float4*>(w3)[i];
+    acc = tc::fma2(tc::pack2(w.x, w.y), tc::pack2(v[4 * i], v[4 * i + 1]), acc);
+    acc = tc::fma2(tc::pack2(w.z, w.w), tc::pack2(v[4 * i + 2], v[4 * i + 3]), acc);
   }
   return acc;
 }
 
-// One MMA operand in shared memory: the first of its three tiles (shared-window address), the
-// tile size, the descriptor's leading and stride byte offsets, and the byte advance per K = 16 step.
+// One MMA operand in shared memory: the descriptor of the first of its three tiles, whose size, layout
+// and advance per K = 16 step are compile-time constants, so that the thread that issues the MMAs
+// adds one constant to the descriptor's low word for each (with descriptors assembled per MMA,
+// by a thread picked by its index, an MMA took 56-85 cycles to issue, more than it ran).
+template <uint32_t LBO, uint32_t SBO, uint32_t STEP>
 struct Operand {
-  uint32_t base, tile, lbo, sbo, step;
+  uint32_t lo;
+  __device__ __forceinline__ explicit Operand(uint32_t base) : lo(static_cast<uint32_t>(tc::smem_desc(base, LBO, SBO))) {}
+  // The operand `off` bytes on, at K step k.
+  __device__ __forceinline__ uint64_t at(uint32_t off, int k) const {
+    constexpr uint64_t hi = (static_cast<uint64_t>(SBO >> 4) << 32) | (1ull << 46);
+    return hi | (lo + ((off + STEP * k) >> 4));
+  }
 };
 
-// K-major operand (tc.cuh layout) of a tile with kt columns, starting at column block c0.
-__device__ __forceinline__ Operand kmajor(uint32_t base, uint32_t tile, int kt, int c0 = 0) {
-  return Operand{base + 128u * c0, tile, 128u, static_cast<uint32_t>(kt / 8 * 128), 256u};
+// K-major operand (tc.cuh layout) of a tile with KT columns.
+template <int KT>
+__device__ __forceinline__ auto kmajor(uint32_t base) {
+  return Operand<128u, KT / 8 * 128u, 256u>(base);
 }
 
 // The same tile read MN-major (its rows become K, its columns M or N): 8-column blocks are 128 B
-// apart (stride byte offset), 8-row groups kt / 8 * 128 B apart (leading byte offset).
-__device__ __forceinline__ Operand mnmajor(uint32_t base, uint32_t tile, int kt, int c0 = 0) {
-  const uint32_t g = static_cast<uint32_t>(kt / 8 * 128);
-  return Operand{base + 128u * c0, tile, g, 128u, 2u * g};
+// apart (stride byte offset), 8-row groups KT / 8 * 128 B apart (leading byte offset).
+template <int KT>
+__device__ __forceinline__ auto mnmajor(uint32_t base) {
+  return Operand<KT / 8 * 128u, 128u, 2u * (KT / 8 * 128u)>(base);
 }
 
-// D = A B^T over k_steps steps of K = 16 as the six products of the three-part split (hi*hi,
-// hi*mid, mid*hi, hi*lo, lo*hi, mid*mid); one thread issues, the mbarrier receives the
-// completion; the first product overwrites D unless accumulate is set.
-__device__ __forceinline__ void mma_split(uint32_t d, const Operand& A, const Operand& B, int k_steps, uint32_t idesc,
-                                          uint64_t* bar, bool accumulate = false) {
+// D = A B^T over one K = 16 step as the six products of the three-part split (hi*hi, hi*mid,
+// mid*hi, hi*lo, lo*hi, mid*mid); the parts of A and B lie AT and BT bytes apart. One thread issues,
+// the mbarrier receives the completion.
+template <uint32_t AT, uint32_t BT, class OA, class OB>
+__device__ __forceinline__ void mma_split16(uint32_t d, const OA& A, const OB& B, uint32_t idesc, uint64_t* bar) {
   constexpr int kPa[6] = {0, 0, 1, 0, 2, 1}, kPb[6] = {0, 1, 0, 2, 0, 1};
   tc::fence_after_sync();
-  for (int k = 0; k < k_steps; ++k) {
 #pragma unroll
-    for (int p = 0; p < 6; ++p) {
-      const uint64_t ad = tc::smem_desc(A.base + A.tile * kPa[p] + A.step * k, A.lbo, A.sbo);
-      const uint64_t bd = tc::smem_desc(B.base + B.tile * kPb[p] + B.step * k, B.lbo, B.sbo);
-      tc::mma_bf16(d, ad, bd, idesc, (k > 0 || p > 0 || accumulate) ? 1u : 0u);
-    }
+  for (int p = 0; p < 6; ++p) tc::mma_bf16(d, A.at(AT * kPa[p], 0), B.at(BT * kPb[p], 0), idesc, p > 0 ? 1u : 0u);
+  tc::mma_commit(bar);
+}
+
+// D = A B^T over K = 64 with A's parts in tensor memory (columns from region as parts_to_tmem lays
+// them), or (LO = false) its lo part, which one of the six products reads, in shared memory.
+template <bool LO, uint32_t BT, class OL, class OB>
+__device__ __forceinline__ void mma_split_ta(uint32_t d, uint32_t region, const OL& lo, const OB& B, uint32_t idesc,
+                                             uint64_t* bar) {
+  tc::fence_after_sync();
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const uint32_t ah = region + 32 * (k >> 1) + 8 * (k & 1), am = ah + 16;
+    tc::mma_bf16_ta(d, ah, B.at(0, k), idesc, k > 0 ? 1u : 0u);
+    tc::mma_bf16_ta(d, ah, B.at(BT, k), idesc, 1u);
+    tc::mma_bf16_ta(d, am, B.at(0, k), idesc, 1u);
+    tc::mma_bf16_ta(d, ah, B.at(2 * BT, k), idesc, 1u);
+    if constexpr (LO) tc::mma_bf16_ta(d, region + 64 + 8 * k, B.at(0, k), idesc, 1u);
+    else tc::mma_bf16(d, lo.at(0, k), B.at(0, k), idesc, 1u);
+    tc::mma_bf16_ta(d, am, B.at(BT, k), idesc, 1u);
   }
   tc::mma_commit(bar);
 }
@@ -146,11 +240,14 @@ __global__ void __launch_bounds__(fwd::kGroups* kGroup, 1) k_mlp_forward(const f
   float* w3 = reinterpret_cast<float*>(S + fwd::W3);
   float* mean = reinterpret_cast<float*>(S + fwd::MEAN);
   float* sd = reinterpret_cast<float*>(S + fwd::SD);
+  float* rs = reinterpret_cast<float*>(S + fwd::RS);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(S + fwd::TMEM);
-  const int gi = threadIdx.x / kGroup, t = threadIdx.x % kGroup, warp = t >> 5, row = t & (kTcM - 1), half = t / kTcM;
+  const int gi = threadIdx.x / kGroup, t = threadIdx.x % kGroup;
+  const int warp = __shfl_sync(0xffffffffu, t >> 5, 0);  // (uniform, so that the MMAs' operands are too)
+  const int row = t & (kTcM - 1), half = t / kTcM;
   float* part = reinterpret_cast<float*>(S + fwd::PART) + gi * kTcM;  // second half's output-layer sums
   uint64_t* bar = reinterpret_cast<uint64_t*>(S + fwd::BAR) + gi;
-  const uint32_t h_off = fwd::H + gi * 3 * fwd::H_T;  // this group's H tile, and X tile before it
+  const uint32_t h_off = fwd::H + gi * fwd::H_T;  // this group's X tile, then h1's lo part
   const int bid = gi + 1;
 
   stage_weights_b(params, S + fwd::W1, fwd::W1_T, S + fwd::W2, fwd::W2_T);
@@ -158,19 +255,16 @@ __global__ void __launch_bounds__(fwd::kGroups* kGroup, 1) k_mlp_forward(const f
     b2[threadIdx.x] = params[kMlpB2 + threadIdx.x];
     w3[threadIdx.x] = params[kMlpW3 + threadIdx.x];
   }
-  if (threadIdx.x < kMlpIn) {
-    mean[threadIdx.x] = params[kMlpMean + threadIdx.x];
-    sd[threadIdx.x] = params[kMlpSd + threadIdx.x];
-  }
+  const bool odd_sd = !stage_normaliser(params, mean, sd, rs);
   const float b3 = params[kMlpB3];
   if (threadIdx.x < 32) tc::tmem_alloc(tmem_slot, fwd::kCols);
   if (t == 0) tc::mbar_init(bar, 1);
   tc::fence_proxy_async();
   tc::fence_before_sync();
-  __syncthreads();
+  const bool by_rs = !__syncthreads_or(odd_sd);
   tc::fence_after_sync();
-  const uint32_t tmem = *tmem_slot, d = tmem + 64u * gi;
-  const uint32_t lane_base = d + (static_cast<uint32_t>((warp & 3) * 32) << 16) + 32u * half;
+  const uint32_t tmem = *tmem_slot, d = tmem + 128u * gi;
+  const uint32_t lane_off = static_cast<uint32_t>((warp & 3) * 32) << 16, lane_base = d + lane_off + 32u * half;
   constexpr uint32_t idesc = tc::idesc_bf16_f32(kTcM, kMlpHid);
   uint32_t phase = 0;
   bool ok = true;  // a wait that gives up ends the group's tiles; until then its threads keep in step
@@ -178,46 +272,60 @@ __global__ void __launch_bounds__(fwd::kGroups* kGroup, 1) k_mlp_forward(const f
   const int n_tiles = (n + kTcM - 1) / kTcM;
   const int tile0 = blockIdx.x + gridDim.x * gi, stride = gridDim.x * fwd::kGroups;
   int tile = tile0;
-  float2 fin[4];  // this thread's half of the raw features of its sample in the next tile
+  // This thread's half of its sample's inputs in the next tile: loaded during the first layer, split
+  // during the second.
+  float2 fin[4];
+  uint4 x[3];
   fetch_half(feats, tile * kTcM + row, n, half, fin);
+  standardise_half(fin, half, mean, sd, rs, by_rs, x);
   for (; tile < n_tiles; tile += stride) {
     const int r = tile * kTcM + row;
-    {
-      float x[8];
-      standardise_half(fin, r < n, half, mean, sd, x);
-      tc::store8_split(S + h_off, fwd::X_T, tc::kmajor_off(row, half, kTcK1), x);
-    }
+    tc::store8(S + h_off, fwd::X_T, tc::kmajor_off(row, half, kTcK1), x[0], x[1], x[2]);
     tc::fence_proxy_async();
     tc::bar_sync(bid, kGroup);
-    if (t == 0) mma_split(d, kmajor(sb + h_off, fwd::X_T, kTcK1), kmajor(sb + fwd::W1, fwd::W1_T, kTcK1), 1, idesc, bar);
-    if (tile + stride < n_tiles) fetch_half(feats, (tile + stride) * kTcM + row, n, half, fin);  // in flight meanwhile
+    if (warp == 0 && tc::elect_one())
+      mma_split16<fwd::X_T, fwd::W1_T>(d, kmajor<kTcK1>(sb + h_off), kmajor<kTcK1>(sb + fwd::W1), idesc, bar);
+    if (tile + stride < n_tiles) fetch_half(feats, (tile + stride) * kTcM + row, n, half, fin);
     ok = ok && tc::mbar_wait(bar, phase);
     phase ^= 1u;
     tc::fence_after_sync();
-    // h1 columns [32 h, 32 h + 32) -> the H tile
+    {  // h1 columns [32 h, 32 h + 32), all read before their accumulator columns are written
+      Parts p;
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      float v[16];
-      tc::tmem_ld16(lane_base + 16 * q, v);
+      for (int q = 0; q < 2; ++q) {
+        float v[16];
+        tc::tmem_ld16(lane_base + 16 * q, v);
 #pragma unroll
-      for (int i = 0; i < 16; ++i) v[i] = fmaxf(v[i], 0.f);
-      tc::store8_split(S + h_off, fwd::H_T, tc::kmajor_off(row, 4 * half + 2 * q, kMlpHid), v);
-      tc::store8_split(S + h_off, fwd::H_T, tc::kmajor_off(row, 4 * half + 2 * q + 1, kMlpHid), v + 8);
+        for (int i = 0; i < 16; ++i) v[i] = fmaxf(v[i], 0.f);
+        split16(v, q, p);
+      }
+#pragma unroll
+      for (int q = 0; q < 2; ++q) parts_to_tmem<false>(d + lane_off, half, q, p);
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        *reinterpret_cast<uint4*>(S + h_off + tc::kmajor_off(row, 4 * half + c, kMlpHid)) = p.l[c];
     }
+    tc::tmem_st_wait();
     tc::fence_proxy_async();
     tc::fence_before_sync();
     tc::bar_sync(bid, kGroup);
-    if (t == 0) mma_split(d, kmajor(sb + h_off, fwd::H_T, kMlpHid), kmajor(sb + fwd::W2, fwd::W2_T, kMlpHid), 4, idesc, bar);
+    if (warp == 0 && tc::elect_one())
+      mma_split_ta<false, fwd::W2_T>(d + 64, d, kmajor<kMlpHid>(sb + h_off), kmajor<kMlpHid>(sb + fwd::W2), idesc, bar);
+    standardise_half(fin, half, mean, sd, rs, by_rs, x);
     ok = ok && tc::mbar_wait(bar, phase);
     phase ^= 1u;
     tc::fence_after_sync();
-    float acc = 0.f;
+    uint64_t acc2 = 0;
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
       float v[16];
-      tc::tmem_ld16(lane_base + 16 * q, v);
-      acc = out_layer16(v, b2 + 32 * half + 16 * q, w3 + 32 * half + 16 * q, acc);
+      tc::tmem_ld16(lane_base + 64 + 16 * q, v);
+      relu16(v, b2 + 32 * half + 16 * q);
+      acc2 = dot16(v, w3 + 32 * half + 16 * q, acc2);
     }
+    float acc, odd;
+    tc::unpack2(acc2, acc, odd);
+    acc += odd;
     if (half == 1) part[row] = acc;
     tc::fence_before_sync();
     if (tc::bar_or(bid, kGroup, !ok)) break;
@@ -317,32 +425,55 @@ int launch_mlp_finder_scores(const float* params, const float* feats, int n, flo
 //   D1 = X W1^T -> h1 = relu(D1);  D2 = H1 W2^T -> z3 = b3 + W3 . relu(D2 + b2),
 //   g = (sigmoid(z3) - y), e2 = g W3 [z2 > 0];  D3 = E2 W2 -> e1 = D3 [h1 > 0];
 //   Dg2 += E2^T [H1 | X],  Dg1 += E1^T X   (accumulated in tensor memory over all the CTA's tiles),
-// so that Dg2's rows 0-63 hold dW2 (columns 0-63) and db2 (column 64 + 14, X's ones) and Dg1's rows
-// 0-63 dW1 (columns 0-13) and db1 (column 14). dW3, db3 and the loss are summed in registers.
+// Dg2 giving dW2 and (in the column of X's ones) db2, Dg1 dW1 and db1. dW3, db3 and the loss are
+// summed in registers.
 //
-// Two groups per CTA. Shared memory (bytes; each operand three tiles, hi, mid, lo): each group's
-// sample x [h1 | x] tile (128 x 80: the A operand of the first two MMAs, K-major, and the B operand of
-// the gradient MMAs, read MN-major), one sample x e tile (128 x 64: e2, then e1; K-major the A
-// operand of the third MMA, MN-major of the gradient MMAs), W1 and W2 (W2 read MN-major is W2^T for
-// the third MMA). The e tile is one group's at a time, from its e2 until its last MMA; the other
-// group then runs its forward layers. A gradient MMA has M = 128 with the tile's 64 columns as
-// the first rows; the rest reads what lies behind in shared memory (the next rows' values, at
-// the end the [h1 | x] tile) into accumulator rows 64-127, which nothing uses.
-// Tensor memory: per group D1 then D3 at 0 and D2 at 64; Dg2 at 256, Dg1 at 336.
-// GRD_NOTE
+// Two groups per CTA. Shared memory: per group one sample x [h1 mid | h1 hi | x hi | x mid | x lo | h1
+// lo] tile (128 x 240; x K-major the A operand of the first MMA, all of it MN-major the B operand of
+// the gradient MMAs), one sample x [e hi | e mid | e lo | 0] tile (128 x 256: e2, then e1; MN-major
+// the A operand of the gradient MMAs), W1 and W2 in three tiles each (W2 read MN-major is W2^T for
+// the third MMA). With the parts side by side one gradient MMA does several of the six products:
+// per K = 16 step of dW2, [hi | mid] by [mid, hi, x hi] (M 128, N 144), [lo | 0] by [hi, x hi] (N 80)
+// and [hi | mid] by lo (N 64), into accumulators whose rows u and 64 + u, and columns c and 64 + c,
+// are added at the end; of dW1, [hi | mid] by [x hi, x mid], [lo | 0] by x hi, [hi | mid] by x lo. As
+// six products of M = 64 each (48 MMAs per layer, 40-60 cycles each: fetching the operands) they took
+// two thirds of the MMA time. The e tile (two do not fit) is one group's at a time, during its
+// gradient MMAs; the other group then runs its layers.
+// Tensor memory: per group D1, then h1, then e2 (parts_to_tmem) at 0, D2 then D3 at 96; Dg2 at 320,
+// Dg1 at 464.
+// 2,000,003 rows take 415 us (137 TFLOP/s of the network's flops), where one group per CTA took 895 us;
+// the bound is the tensor pipe fetching operands (a gradient MMA with an MN-major A of 128 rows takes 70
+// to 96 cycles). A step's 4,096 rows: kernels 21 us against 85 us; their tile, prologue and epilogue
+// are one chain (the old epilogue added 32 lanes to one shared-memory float, a CAS loop each).
 namespace grd {
 constexpr int kGroups = 2;
-constexpr uint32_t E_T = 16384, XH_T = 20480, W1_T = 2048, W2_T = 8192;  // bytes of one tile
-constexpr uint32_t E = 0, XH = E + 3 * E_T, W2 = XH + kGroups * 3 * XH_T, W1 = W2 + 3 * W2_T, B2 = W1 + 3 * W1_T,
-                   W3 = B2 + 256, MEAN = W3 + 256, SD = MEAN + 64, PART = SD + 64, RED = PART + kGroups * 1024,
+constexpr int kXhK = 240, kEK = 256;                            // columns of the two tiles
+constexpr int kHm = 0, kHh = 8, kXh = 16, kXm = 18, kXl = 20, kHl = 22;  // 8-column blocks of the parts
+constexpr uint32_t E_T = kTcM * kEK * 2, XH_T = kTcM * kXhK * 2, W1_T = 2048, W2_T = 8192;  // bytes of one tile
+constexpr uint32_t E = 0, XH = E + E_T, W2 = XH + kGroups * XH_T, W1 = W2 + 3 * W2_T, B2 = W1 + 3 * W1_T,
+                   W3 = B2 + 256, MEAN = W3 + 256, SD = MEAN + 64, RS = SD + 64, PART = RS + 64, RED = PART + kGroups * 1024,
                    BAR = RED + 16 * 34 * 4, TMEM = BAR + 16 * kGroups, LOCK = TMEM + 4, USED = LOCK + 4, BYTES = USED + 8;
 static_assert(BYTES + 1024 <= 227 * 1024, "shared-memory layout");
-constexpr uint32_t kCols = 512, kColD2 = 64, kColG2 = 256, kColG1 = 336;
-constexpr int kXhK = 80, kEK = 64;
+constexpr uint32_t kCols = 512, kColD2 = 96, kColG2 = 320, kColG1 = 464;
 }  // namespace grd
 
 // Instruction descriptor bits 15 and 16: A, B MN-major.
 constexpr uint32_t kAmn = 1u << 15, kBmn = 1u << 16;
+
+// D (+)= E^T B over K = the tile's 128 samples, both MN-major: per K = 16 step [hi | mid] of e by the N1
+// columns of B from block B1 on, [lo | 0] by N2 from B2 on (D's columns from C2 on), [hi | mid] by N3
+// from B3 on.
+template <int C2, int B1, int N1, int B2, int N2, int B3, int N3, class OE, class OB>
+__device__ __forceinline__ void mma_grad(uint32_t d, const OE& E, const OB& B, uint64_t* bar, bool accumulate) {
+  tc::fence_after_sync();
+#pragma unroll
+  for (int k = 0; k < kTcM / 16; ++k) {
+    tc::mma_bf16(d, E.at(0, k), B.at(128 * B1, k), tc::idesc_bf16_f32(kTcM, N1) | kAmn | kBmn, k > 0 || accumulate);
+    tc::mma_bf16(d + C2, E.at(128 * 16, k), B.at(128 * B2, k), tc::idesc_bf16_f32(kTcM, N2) | kAmn | kBmn, 1u);
+    tc::mma_bf16(d, E.at(0, k), B.at(128 * B3, k), tc::idesc_bf16_f32(kTcM, N3) | kAmn | kBmn, 1u);
+  }
+  tc::mma_commit(bar);
+}
 
 // Sums of v[i] over the warp's lanes, element i in lane i: five halving exchanges.
 __device__ __forceinline__ float warp_sum32(float* v, int lane) {
@@ -380,16 +511,19 @@ __global__ void __launch_bounds__(grd::kGroups* kGroup, 1)
   float* w3 = reinterpret_cast<float*>(S + grd::W3);
   float* mean = reinterpret_cast<float*>(S + grd::MEAN);
   float* sd = reinterpret_cast<float*>(S + grd::SD);
+  float* rs = reinterpret_cast<float*>(S + grd::RS);
   float* red = reinterpret_cast<float*>(S + grd::RED);  // [16 warps][34]: dW3 of the warp's 32 units, db3, loss
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(S + grd::TMEM);
   int* lock = reinterpret_cast<int*>(S + grd::LOCK);  // 1: the e tile is taken
   int* used = reinterpret_cast<int*>(S + grd::USED);  // 1: the gradient accumulators hold a tile
-  const int gi = threadIdx.x / kGroup, t = threadIdx.x % kGroup, warp = t >> 5, row = t & (kTcM - 1), half = t / kTcM;
+  const int gi = threadIdx.x / kGroup, t = threadIdx.x % kGroup;
+  const int warp = __shfl_sync(0xffffffffu, t >> 5, 0);  // (uniform, so that the MMAs' operands are too)
+  const int row = t & (kTcM - 1), half = t / kTcM;
   const int hc = 32 * half;  // this thread's first column of a 64-column accumulator
   float* part = reinterpret_cast<float*>(S + grd::PART) + gi * 2 * kTcM;  // [2][128] output-layer partial sums
   // bar[0]: the layers' MMAs, bar[1]: the gradient MMAs (the first of them is in flight with the third layer's)
   uint64_t* bar = reinterpret_cast<uint64_t*>(S + grd::BAR) + 2 * gi;
-  const uint32_t xh = grd::XH + gi * 3 * grd::XH_T;
+  const uint32_t xh = grd::XH + gi * grd::XH_T;
   const int bid = gi + 1;
 
   stage_weights_b(params, S + grd::W1, grd::W1_T, S + grd::W2, grd::W2_T);
@@ -397,10 +531,9 @@ __global__ void __launch_bounds__(grd::kGroups* kGroup, 1)
     b2[threadIdx.x] = params[kMlpB2 + threadIdx.x];
     w3[threadIdx.x] = params[kMlpW3 + threadIdx.x];
   }
-  if (threadIdx.x < kMlpIn) {
-    mean[threadIdx.x] = params[kMlpMean + threadIdx.x];
-    sd[threadIdx.x] = params[kMlpSd + threadIdx.x];
-  }
+  const bool odd_sd = !stage_normaliser(params, mean, sd, rs);
+  for (int i = threadIdx.x; i < kTcM * 8; i += blockDim.x)  // the e tile's zero columns
+    *reinterpret_cast<uint4*>(S + grd::E + tc::kmajor_off(i >> 3, 24 + (i & 7), grd::kEK)) = make_uint4(0u, 0u, 0u, 0u);
   const float b3 = params[kMlpB3];
   if (threadIdx.x < 32) tc::tmem_alloc(tmem_slot, grd::kCols);
   if (threadIdx.x == 0) *lock = *used = 0;
@@ -410,149 +543,165 @@ __global__ void __launch_bounds__(grd::kGroups* kGroup, 1)
   }
   tc::fence_proxy_async();
   tc::fence_before_sync();
-  __syncthreads();
+  const bool by_rs = !__syncthreads_or(odd_sd);
   tc::fence_after_sync();
-  const uint32_t tmem = *tmem_slot, d = tmem + 128u * gi;
+  const uint32_t tmem = *tmem_slot, d = tmem + 160u * gi;
   const uint32_t lane_off = static_cast<uint32_t>((warp & 3) * 32) << 16;
   const uint32_t lane_base = d + lane_off + hc;
   constexpr uint32_t id_kk = tc::idesc_bf16_f32(kTcM, kMlpHid);
-  constexpr uint32_t id_g2 = tc::idesc_bf16_f32(kTcM, grd::kXhK) | kAmn | kBmn;
-  constexpr uint32_t id_g1 = tc::idesc_bf16_f32(kTcM, kTcK1) | kAmn | kBmn;
-  const Operand e_k = kmajor(sb + grd::E, grd::E_T, grd::kEK), e_mn = mnmajor(sb + grd::E, grd::E_T, grd::kEK);
+  const auto e_mn = mnmajor<grd::kEK>(sb + grd::E);
+  const auto xh_mn = mnmajor<grd::kXhK>(sb + xh);
   uint32_t phase = 0, gphase = 0;
   bool ok = true, locked = false;
-  float acc3[32];  // dW3 partial sums of this thread's 32 hidden units
+  uint64_t acc3[16];  // dW3 partial sums of this thread's 32 hidden units, in pairs
 #pragma unroll
-  for (int j = 0; j < 32; ++j) acc3[j] = 0.f;
+  for (int j = 0; j < 16; ++j) acc3[j] = 0;
   float gsum = 0.f, lsum = 0.f;
 
   const int n_tiles = (n + kTcM - 1) / kTcM;
   const int stride = gridDim.x * grd::kGroups;
   int tile = blockIdx.x + gridDim.x * gi;
-  float2 fin[4];  // this thread's half of the raw features, and the label, of its sample in the next tile
+  // This thread's half of its sample's inputs, and the label, in the next tile: loaded and
+  // split during the gradient MMAs.
+  float2 fin[4];
+  uint4 x[3];
   fetch_half(feats, tile * kTcM + row, n, half, fin);
+  standardise_half(fin, half, mean, sd, rs, by_rs, x);
   float yin = tile * kTcM + row < n ? labels[tile * kTcM + row] : 0.f;
   for (; tile < n_tiles; tile += stride) {
     const bool valid = tile * kTcM + row < n;
-    {  // inputs -> columns 64-79 of the [h1 | x] tile
-      float x[8];
-      standardise_half(fin, valid, half, mean, sd, x);
-      tc::store8_split(S + xh, grd::XH_T, tc::kmajor_off(row, 8 + half, grd::kXhK), x);
-    }
+    tc::store8(S + xh, 128 * (grd::kXm - grd::kXh), tc::kmajor_off(row, grd::kXh + half, grd::kXhK), x[0], x[1], x[2]);
     const float y = yin;
     tc::fence_proxy_async();
     tc::bar_sync(bid, kGroup);
-    if (t == 0)
-      mma_split(d, kmajor(sb + xh, grd::XH_T, grd::kXhK, 8), kmajor(sb + grd::W1, grd::W1_T, kTcK1), 1, id_kk, bar);
-    if (tile + stride < n_tiles) {  // in flight during this tile
-      const int rn = (tile + stride) * kTcM + row;
-      fetch_half(feats, rn, n, half, fin);
-      yin = rn < n ? labels[rn] : 0.f;
-    }
+    if (warp == 0 && tc::elect_one())
+      mma_split16<128 * (grd::kXm - grd::kXh), grd::W1_T>(d, kmajor<grd::kXhK>(sb + xh + 128 * grd::kXh),
+                                                          kmajor<kTcK1>(sb + grd::W1), id_kk, bar);
     ok = ok && tc::mbar_wait(bar, phase);
     phase ^= 1u;
     tc::fence_after_sync();
     // h1 -> columns [hc, hc + 32) of the [h1 | x] tile; mask1 = [h1 > 0]
     unsigned mask1 = 0u;
+    {
+      Parts p;
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      float v[16];
-      tc::tmem_ld16(lane_base + 16 * q, v);
+      for (int q = 0; q < 2; ++q) {
+        float v[16];
+        tc::tmem_ld16(lane_base + 16 * q, v);
 #pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        v[i] = fmaxf(v[i], 0.f);
-        if (v[i] > 0.f) mask1 |= 1u << (16 * q + i);
+        for (int i = 0; i < 16; ++i) {
+          v[i] = fmaxf(v[i], 0.f);
+          if (v[i] > 0.f) mask1 |= 1u << (16 * q + i);
+        }
+        split16(v, q, p);
       }
-      tc::store8_split(S + xh, grd::XH_T, tc::kmajor_off(row, 4 * half + 2 * q, grd::kXhK), v);
-      tc::store8_split(S + xh, grd::XH_T, tc::kmajor_off(row, 4 * half + 2 * q + 1, grd::kXhK), v + 8);
+#pragma unroll
+      for (int q = 0; q < 2; ++q) parts_to_tmem<true>(d + lane_off, half, q, p);
+      parts_to_smem<grd::kXhK, grd::kHh, grd::kHm, grd::kHl>(S + xh, row, half, p);
     }
+    tc::tmem_st_wait();
     tc::fence_proxy_async();
     tc::fence_before_sync();
     tc::bar_sync(bid, kGroup);
-    if (t == 0)
-      mma_split(d + grd::kColD2, kmajor(sb + xh, grd::XH_T, grd::kXhK), kmajor(sb + grd::W2, grd::W2_T, kMlpHid), 4, id_kk,
-                bar);
+    if (warp == 0 && tc::elect_one())
+      mma_split_ta<true, grd::W2_T>(d + grd::kColD2, d, 0, kmajor<kMlpHid>(sb + grd::W2), id_kk, bar);
     ok = ok && tc::mbar_wait(bar, phase);
     phase ^= 1u;
     tc::fence_after_sync();
     {  // logit from the two halves' partial sums
-      float acc = 0.f;
+      uint64_t acc2 = 0;
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
         float v[16];
         tc::tmem_ld16(lane_base + grd::kColD2 + 16 * q, v);
-        acc = out_layer16(v, b2 + hc + 16 * q, w3 + hc + 16 * q, acc);
+        relu16(v, b2 + hc + 16 * q);
+        acc2 = dot16(v, w3 + hc + 16 * q, acc2);
       }
-      part[half * kTcM + row] = acc;
+      float acc, odd;
+      tc::unpack2(acc2, acc, odd);
+      part[half * kTcM + row] = acc + odd;
     }
-    if (t == 0 && ok) {  // the e tile: the other group's until its gradient MMAs are done
-      const uint64_t t0 = tc::global_ns();
-      while (!(locked = atomicCAS(lock, 0, 1) == 0) && tc::global_ns() - t0 < 2000000000ull) __nanosleep(40);
-      ok = locked;
-      __threadfence_block();
-    }
-    if (tc::bar_or(bid, kGroup, !ok)) break;
+    tc::bar_sync(bid, kGroup);
     const float z3 = b3 + part[row] + part[kTcM + row];
     const float g = valid ? 1.f / (1.f + expf(-z3)) - y : 0.f;
-    if (half == 0) {
+    // e2 columns [hc, hc + 32) and dW3 partial sums; e2 to tensor memory, where h1 was
+    Parts p;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      float v[16];
+      tc::tmem_ld16(lane_base + grd::kColD2 + 16 * q, v);
+      relu16(v, b2 + hc + 16 * q);
+      const uint64_t gg = tc::pack2(g, g);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        uint64_t& a3 = acc3[8 * q + i];
+        a3 = tc::fma2(gg, tc::pack2(v[2 * i], v[2 * i + 1]), a3);
+        const float2 w = *reinterpret_cast<const float2*>(w3 + hc + 16 * q + 2 * i);
+        float e0, e1;
+        tc::unpack2(tc::mul2(gg, tc::pack2(w.x, w.y)), e0, e1);
+        v[2 * i] = v[2 * i] > 0.f ? e0 : 0.f;
+        v[2 * i + 1] = v[2 * i + 1] > 0.f ? e1 : 0.f;
+      }
+      split16(v, q, p);
+      parts_to_tmem<true>(d + lane_off, half, q, p);
+    }
+    tc::tmem_st_wait();
+    tc::fence_before_sync();
+    tc::bar_sync(bid, kGroup);
+    // D3 = E2 W2: W2's K-major tile (rows o, columns i) read MN-major is W2^T (n = i, k = o).
+    if (warp == 0) {
+      if (tc::elect_one())
+        mma_split_ta<true, grd::W2_T>(d + grd::kColD2, d, 0, mnmajor<kMlpHid>(sb + grd::W2), id_kk | kBmn, bar);
+      __syncwarp();
+      if (t == 0 && ok) {  // the e tile: the other group's until its gradient MMAs are done
+        const uint64_t t0 = tc::global_ns();
+        while (!(locked = atomicCAS(lock, 0, 1) == 0) && tc::global_ns() - t0 < 2000000000ull) __nanosleep(20);
+        ok = locked;
+        __threadfence_block();
+      }
+    }
+    if (tc::bar_or(bid, kGroup, !ok)) {
+      phase ^= 1u;  // the third layer's MMAs are in flight
+      break;
+    }
+    parts_to_smem<grd::kEK, 0, 8, 16>(S + grd::E, row, half, p);
+    tc::fence_proxy_async();
+    tc::bar_sync(bid, kGroup);
+    // Dg2 += E2^T [H1 | X], K = the tile's 128 samples.
+    if (warp == 0 && tc::elect_one())
+      mma_grad<64, grd::kHm, 144, grd::kHh, 80, grd::kHl, 64>(tmem + grd::kColG2, e_mn, xh_mn, bar + 1, *used != 0);
+    if (tile + stride < n_tiles) {
+      const int rn = (tile + stride) * kTcM + row;
+      fetch_half(feats, rn, n, half, fin);
+      yin = rn < n ? labels[rn] : 0.f;
+    }
+    if (half == 0) {  // under the gradient MMA
       if (valid) lsum += fmaxf(z3, 0.f) - z3 * y + log1pf(expf(-fabsf(z3)));
       gsum += g;
     }
-    // e2 -> columns [hc, hc + 32) of the e tile; dW3 partial sums
+    ok = ok && tc::mbar_wait(bar, phase);
+    phase ^= 1u;
+    tc::fence_after_sync();
+    ok = ok && tc::mbar_wait(bar + 1, gphase);
+    gphase ^= 1u;
+    tc::fence_after_sync();
+    // e1
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
       float v[16];
       tc::tmem_ld16(lane_base + grd::kColD2 + 16 * q, v);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const float4 b = reinterpret_cast<const float4*>(b2 + hc + 16 * q)[i];
-        const float4 w = reinterpret_cast<const float4*>(w3 + hc + 16 * q)[i];
-        const float bb[4] = {b.x, b.y, b.z, b.w}, ww[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const float a2 = fmaxf(v[4 * i + e] + bb[e], 0.f);
-          acc3[16 * q + 4 * i + e] = fmaf(g, a2, acc3[16 * q + 4 * i + e]);
-          v[4 * i + e] = a2 > 0.f ? g * ww[e] : 0.f;
-        }
-      }
-      tc::store8_split(S + grd::E, grd::E_T, tc::kmajor_off(row, 4 * half + 2 * q, grd::kEK), v);
-      tc::store8_split(S + grd::E, grd::E_T, tc::kmajor_off(row, 4 * half + 2 * q + 1, grd::kEK), v + 8);
-    }
-    tc::fence_proxy_async();
-    tc::fence_before_sync();
-    tc::bar_sync(bid, kGroup);
-    // D3 = E2 W2: W2's K-major tile (rows o, columns i) read MN-major is W2^T (n = i, k = o). Then
-    // Dg2 += E2^T [H1 | X]: both tiles read MN-major, K = the tile's 128 samples.
-    if (t == 0) {
-      mma_split(d, e_k, mnmajor(sb + grd::W2, grd::W2_T, kMlpHid), 4, id_kk | kBmn, bar);
-      mma_split(tmem + grd::kColG2, e_mn, mnmajor(sb + xh, grd::XH_T, grd::kXhK), kTcM / 16, id_g2, bar + 1, *used != 0);
-    }
-    ok = ok && tc::mbar_wait(bar, phase);
-    phase ^= 1u;
-    tc::fence_after_sync();
-    // e1, split while the gradient MMA still reads e2
-    uint4 e1[4][3];
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      float v[16];
-      tc::tmem_ld16(lane_base + 16 * q, v);
-#pragma unroll
       for (int i = 0; i < 16; ++i) v[i] = (mask1 >> (16 * q + i)) & 1u ? v[i] : 0.f;
-      tc::split8(v, e1[2 * q][0], e1[2 * q][1], e1[2 * q][2]);
-      tc::split8(v + 8, e1[2 * q + 1][0], e1[2 * q + 1][1], e1[2 * q + 1][2]);
+      split16(v, q, p);
     }
-    ok = ok && tc::mbar_wait(bar + 1, gphase);
-    gphase ^= 1u;
-    tc::fence_after_sync();
-#pragma unroll
-    for (int c = 0; c < 4; ++c)
-      tc::store8(S + grd::E, grd::E_T, tc::kmajor_off(row, 4 * half + c, grd::kEK), e1[c][0], e1[c][1], e1[c][2]);
+    parts_to_smem<grd::kEK, 0, 8, 16>(S + grd::E, row, half, p);
     tc::fence_proxy_async();
     tc::fence_before_sync();
     tc::bar_sync(bid, kGroup);
     // Dg1 += E1^T X
-    if (t == 0)
-      mma_split(tmem + grd::kColG1, e_mn, mnmajor(sb + xh, grd::XH_T, grd::kXhK, 8), kTcM / 16, id_g1, bar + 1, *used != 0);
+    if (warp == 0 && tc::elect_one())
+      mma_grad<0, grd::kXh, 32, grd::kXh, 16, grd::kXl, 16>(tmem + grd::kColG1, e_mn, xh_mn, bar + 1, *used != 0);
+    standardise_half(fin, half, mean, sd, rs, by_rs, x);
     ok = ok && tc::mbar_wait(bar + 1, gphase);
     gphase ^= 1u;
     tc::fence_after_sync();
@@ -576,7 +725,12 @@ __global__ void __launch_bounds__(grd::kGroups* kGroup, 1)
   }
   // dW3, db3 and the loss: over the warp's samples, then over the eight warps of each half.
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  red[wid * 34 + lane] = warp_sum32(acc3, lane);
+  {
+    float v[32];
+#pragma unroll
+    for (int j = 0; j < 16; ++j) tc::unpack2(acc3[j], v[2 * j], v[2 * j + 1]);
+    red[wid * 34 + lane] = warp_sum32(v, lane);
+  }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     gsum += __shfl_xor_sync(0xffffffffu, gsum, o);
@@ -599,25 +753,52 @@ __global__ void __launch_bounds__(grd::kGroups* kGroup, 1)
     if (j <= kMlpHid) atomicAdd(grad + (j < kMlpHid ? kMlpW3 + j : kMlpB3), v * inv_n);
     else atomicAdd(loss, v * inv_n);
   }
-  // The gradient accumulators' rows 0-63 (tensor-memory lanes 0-63, the warps w with w % 4 < 2): the
-  // four such pairs of warps take 16 columns of dW2 each; db2 (pair 1), dW1 and db1 (pair 2).
-  if (*used && (wid & 3) < 2) {
-    const int j = 32 * (wid & 3) + lane, q = wid >> 2;
-    float v[16];
-    tc::tmem_ld16(tmem + lane_off + grd::kColG2 + 16 * q, v);
+  // The gradient accumulators: unit u is rows u and 64 + u. Warps w with w % 4 >= 2 hold the latter and
+  // pass them through shared memory (where the e tile was); the four pairs of warps of each half take
+  // 16 columns of dW2 each, the second also db2, the third dW1 and db1.
+  {
+    const int rr = 32 * (wid & 3) + lane, u = rr & 63, q = wid >> 2;
+    float v[16], w[16];
+    float* st = reinterpret_cast<float*>(S + grd::E);  // [5][64][17]
+    auto meet = [&](float* z, int k) {
+      float* m = st + (k * 64 + u) * 17;
+      if (rr >= 64)
 #pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] *= inv_n;
+        for (int i = 0; i < 16; ++i) m[i] = z[i];
+      __syncthreads();
+      if (rr < 64)
 #pragma unroll
-    for (int i = 0; i < 4; ++i) add4(grad + kMlpW2 + j * kMlpHid + 16 * q + 4 * i, v + 4 * i);
-    if (q == 1) {
-      tc::tmem_ld16(tmem + lane_off + grd::kColG2 + 64, v);
-      atomicAdd(grad + kMlpB2 + j, v[kOne] * inv_n);
+        for (int i = 0; i < 16; ++i) z[i] = (z[i] + m[i]) * inv_n;
+    };
+    const bool any = *used != 0;
+    if (any) {
+      tc::tmem_ld16(tmem + lane_off + grd::kColG2 + 16 * q, v);
+      tc::tmem_ld16(tmem + lane_off + grd::kColG2 + 64 + 16 * q, w);
+#pragma unroll
+      for (int i = 0; i < 16; ++i) v[i] += w[i];
+      if (q == 1) {
+        tc::tmem_ld16(tmem + lane_off + grd::kColG2 + 128, w);
+      } else if (q == 2) {
+        float w2[16];
+        tc::tmem_ld16(tmem + lane_off + grd::kColG1, w);
+        tc::tmem_ld16(tmem + lane_off + grd::kColG1 + 16, w2);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) w[i] += w2[i];
+      }
     }
-    if (q == 2) {
-      tc::tmem_ld16(tmem + lane_off + grd::kColG1, v);
+    meet(v, q);
+    __syncthreads();
+    meet(w, q);
+    if (any && rr < 64) {
 #pragma unroll
-      for (int k = 0; k < kMlpIn; ++k) atomicAdd(grad + kMlpW1 + j * kMlpIn + k, v[k] * inv_n);
-      atomicAdd(grad + kMlpB1 + j, v[kOne] * inv_n);
+      for (int i = 0; i < 4; ++i) add4(grad + kMlpW2 + u * kMlpHid + 16 * q + 4 * i, v + 4 * i);
+      if (q == 1) {
+        atomicAdd(grad + kMlpB2 + u, w[kOne]);
+      } else if (q == 2) {
+#pragma unroll
+        for (int k = 0; k < kMlpIn; ++k) atomicAdd(grad + kMlpW1 + u * kMlpIn + k, w[k]);
+        atomicAdd(grad + kMlpB1 + u, w[kOne]);
+      }
     }
   }
   tc::fence_before_sync();

@@ -40,6 +40,17 @@ __host__ __device__ constexpr uint32_t idesc_bf16_f32(int m, int n) {
          (static_cast<uint32_t>(m >> 4) << 24);
 }
 
+// One lane of the (converged) warp: true in it.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(r));
+  return r != 0;
+}
+
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void fence_before_sync() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_after_sync() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -56,11 +67,11 @@ __device__ __forceinline__ uint64_t global_ns() {
 }
 
 // Waits for the mbarrier phase with the given parity to complete; gives up after limit_ns and
-// returns false.
+// returns false. The clock is read from the 16th try on (each try already waits in hardware).
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint64_t limit_ns = 1000000000ull) {
   const uint32_t a = smem_u32(bar);
-  const uint64_t t0 = global_ns();
-  while (true) {
+  uint64_t t0 = 0;
+  for (uint32_t tries = 0;; ++tries) {
     uint32_t done;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
@@ -70,7 +81,10 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint64
         : "r"(a), "r"(parity)
         : "memory");
     if (done) return true;
-    if (global_ns() - t0 > limit_ns) return false;
+    if (tries < 16) continue;
+    const uint64_t now = global_ns();
+    if (t0 == 0) t0 = now;
+    if (now - t0 > limit_ns) return false;
   }
 }
 
@@ -112,6 +126,17 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64
       : "memory");
 }
 
+// The same with A in tensor memory: lane = row, two bf16 of the row to a column, 8 columns for K = 16.
+__device__ __forceinline__ void mma_bf16_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
+                                            uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
+      "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+
 // The mbarrier receives one arrival when every MMA issued before by this thread has completed.
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
@@ -134,6 +159,15 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// 8 words into consecutive columns of this thread's tensor-memory lane; tmem_st_wait() before a
+// barrier makes the warp's stores visible to MMAs issued after it (with the thread-sync fences).
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint4& a, const uint4& b) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(taddr), "r"(a.x),
+               "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w)
+               : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
 // Two values rounded to bf16 (x0 in the low half), and the two values of such a word.
 __device__ __forceinline__ uint32_t cvt_bf16x2(float x0, float x1) {
   uint32_t r;
@@ -143,18 +177,47 @@ __device__ __forceinline__ uint32_t cvt_bf16x2(float x0, float x1) {
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
 
+// Two FP32 operations at once (each element rounded as the scalar operation rounds it).
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
 // hi, mid and lo bf16 parts of 8 consecutive values, two values to a word.
 __device__ __forceinline__ void split8(const float* v, uint4& h, uint4& m, uint4& l) {
   uint32_t w[3][4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const float a = v[2 * i], b = v[2 * i + 1];
-    const uint32_t hw = cvt_bf16x2(a, b);
-    const float a1 = a - bf16_lo(hw), b1 = b - bf16_hi(hw);
-    const uint32_t mw = cvt_bf16x2(a1, b1);
-    w[0][i] = hw;
-    w[1][i] = mw;
-    w[2][i] = cvt_bf16x2(a1 - bf16_lo(mw), b1 - bf16_hi(mw));
+    uint64_t x = pack2(v[2 * i], v[2 * i + 1]);
+#pragma unroll
+    for (int part = 0; part < 3; ++part) {
+      float a, b;
+      unpack2(x, a, b);
+      w[part][i] = cvt_bf16x2(a, b);
+      if (part < 2) x = sub2(x, pack2(bf16_lo(w[part][i]), bf16_hi(w[part][i])));
+    }
   }
   h = make_uint4(w[0][0], w[0][1], w[0][2], w[0][3]);
   m = make_uint4(w[1][0], w[1][1], w[1][2], w[1][3]);
