@@ -14,6 +14,10 @@ namespace kfgb {
 __global__ void k_build_hit_index(DevGeom G, const float2* hits, const int* slab_off, int n_slabs, int cap,
                                   int* bin_off, float2* sorted_hits, int* sorted_ids, float4* sorted_rec,
                                   uint4* sub_off, int* d_status);
+__global__ void k_build_hit_index_fine(const __grid_constant__ DevGeom G, const float2* hits, const int* slab_off,
+                                       int n_slabs, int cap, int* bin_off, float2* sorted_hits, int* sorted_ids,
+                                       float4* sorted_rec, uint4* sub_off, int* d_status);
+constexpr int kFineMaxBins = 8192;  // hitindex.cu
 __global__ void k_fit_tracks(DevGeom G, const __grid_constant__ DevMat M, const float2* hits, const int* hit_surface,
                              const int* track_hits,
                              int n_tracks, int lmax, float* state_out, float* cov_out, float* chi2_out, int* ndof_out,
@@ -226,23 +230,34 @@ int kf_build_hit_index(const KfGeometry* geom, const float* hits, const int* sla
     return KF_ERR_ARG;
   const int n_slabs = n_events * G.n_surf;
   const int cap = std::max(2, (max_slab_hits + 1) & ~1);
-  const size_t smem = static_cast<size_t>(G.n_bins + 1) * sizeof(int) + 2 * static_cast<size_t>(cap) * sizeof(unsigned short) +
-                      static_cast<size_t>(cap) * sizeof(unsigned char);
+  // Fine bins where a fine bin fits 16 bits and two blocks still share an SM (or the other kernel's
+  // blocks do not either); else the kernel with bins and sub-bins apart, which takes 4 bytes a bin
+  // and 5 a hit of shared memory instead of 16 and 4.
+  const size_t by_bins = static_cast<size_t>(G.n_bins + 1) * sizeof(int) + 5 * static_cast<size_t>(cap);
+  const size_t by_fine = static_cast<size_t>(G.n_bins) * 16 + 4 * static_cast<size_t>(cap);
+  constexpr size_t kHalf = 113 * 1024, kAll = 226 * 1024;
+  const bool fine = G.n_bins <= kFineMaxBins && (by_fine <= kHalf || (by_bins > kHalf && by_fine <= kAll));
+  const size_t smem = fine ? by_fine : by_bins;
   // Raise the kernel's dynamic shared memory limit once per device (and only when a larger slab
   // needs it), so later calls, e.g. inside a stream capture, make no attribute call.
-  static int smem_set[64] = {0};
+  static int smem_set[2][64] = {{0}};
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return KF_ERR_CUDA;
-  if (static_cast<int>(smem) > smem_set[dev]) {
-    if (cudaFuncSetAttribute(k_build_hit_index, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(smem)) != cudaSuccess)
-      return KF_ERR_CUDA;
-    smem_set[dev] = static_cast<int>(smem);
+  if (static_cast<int>(smem) > smem_set[fine][dev]) {
+    const cudaError_t e =
+        fine ? cudaFuncSetAttribute(k_build_hit_index_fine, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem))
+             : cudaFuncSetAttribute(k_build_hit_index, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (e != cudaSuccess) return KF_ERR_CUDA;
+    smem_set[fine][dev] = static_cast<int>(smem);
   }
-  k_build_hit_index<<<n_slabs, 1024, smem, reinterpret_cast<cudaStream_t>(stream)>>>(
-      G, reinterpret_cast<const float2*>(hits), slab_offsets, n_slabs, cap, index->bin_off,
-      reinterpret_cast<float2*>(index->sorted_hits), index->sorted_ids, reinterpret_cast<float4*>(index->sorted_rec),
-      reinterpret_cast<uint4*>(index->sub_off), d_status);
+  auto launch = [&](auto kernel) {
+    kernel<<<n_slabs, 1024, smem, reinterpret_cast<cudaStream_t>(stream)>>>(
+        G, reinterpret_cast<const float2*>(hits), slab_offsets, n_slabs, cap, index->bin_off,
+        reinterpret_cast<float2*>(index->sorted_hits), index->sorted_ids, reinterpret_cast<float4*>(index->sorted_rec),
+        reinterpret_cast<uint4*>(index->sub_off), d_status);
+  };
+  if (fine) launch(k_build_hit_index_fine);
+  else launch(k_build_hit_index);
   return launch_status();
 }
 
