@@ -48,20 +48,14 @@ struct WarpSmem {
   float4 win_a[32];        // window of each lane: x, y, centre of the 2nd coordinate, transverse scale
   float4 win_b[32];        // S^-1 (00, 01, 11) and the far-hit threshold of window_chi2
   int2 rows[kRows][32];    // runs: (end of the run in the lane's flattened window, position - start)
-  float hl_tot[KC][32];    // per lane: best passing hits, sorted by (total chi2, hit id)
-  int hl_id[KC][32];
-  int hl_pos[KC][32];
+  float hl_tot[KC][32];    // per lane: best passing hits, sorted by (total chi2, hit id), and their
+  int hl_pos[KC][32];      // positions in the index (the record there holds the id)
   unsigned long long tab_key[32];  // winner table of each group, by rank
-  int tab_id[32];
   int tab_pos[32];
-  union {
-    struct {
-      float c2[kPList];
-      int id[kPList];
-      int pos[kPList];
-      int own[kPList];
-    } pl;                               // buffered passing pairs (scan)
-  } u;
+  struct {
+    float c2[kPList];
+    int pos[kPList];
+  } pl;  // buffered passing pairs (scan)
 };
 
 // Learned instances of up to 4 slots hold the network's weight fragments in shared memory, after
@@ -90,51 +84,55 @@ __host__ __device__ size_t warp_smem_bytes(int lmax) {
           (LEARNED ? sizeof(WarpLearned<KC>) : 0) + 15) / 16 * 16;
 }
 
-__device__ __forceinline__ bool before(float t, int id, float u, int uid) { return t < u || (t == u && id < uid); }
+// Hit id at a position of the index (inverted positions: see window ranking). The lists keep positions
+// only (768-1,024 B of shared memory per warp less: two more warps per SM at 8 slots); ids break the
+// rare ties.
+__device__ __forceinline__ int id_at(const float4* __restrict__ rec, int pos) {
+  return __float_as_int(__ldg(&rec[pos < 0 ? ~pos : pos].w));
+}
+__device__ __forceinline__ bool before(const float4* __restrict__ rec, float t, int pos, float u, int upos) {
+  return t < u || (t == u && id_at(rec, pos) < id_at(rec, upos));
+}
 
 // Insert into a lane's kept list ordered by (score descending, hit id ascending), capacity cap.
 template <int KC>
-__device__ __forceinline__ void hl_insert_scored(WarpSmem<KC>& W, WarpLearned<KC>& L, int lane, int& n, int cap,
-                                                 float sc, float tot, int id, int pos) {
+__device__ __forceinline__ void hl_insert_scored(WarpSmem<KC>& W, WarpLearned<KC>& L, const float4* __restrict__ rec,
+                                                 int lane, int& n, int cap, float sc, float tot, int pos) {
+  auto ahead = [&](int i) {  // of entry i
+    const float s = L.hl_sc[i][lane];
+    return sc > s || (sc == s && id_at(rec, pos) < id_at(rec, W.hl_pos[i][lane]));
+  };
   if (n == cap) {
-    const float ls = L.hl_sc[cap - 1][lane];
-    const int li = W.hl_id[cap - 1][lane];
-    if (!(sc > ls || (sc == ls && id < li))) return;
+    if (!ahead(cap - 1)) return;
     n = cap - 1;
   }
   int i = n;
-  while (i > 0) {
-    const float ps = L.hl_sc[i - 1][lane];
-    const int pi = W.hl_id[i - 1][lane];
-    if (!(sc > ps || (sc == ps && id < pi))) break;
-    L.hl_sc[i][lane] = ps;
+  while (i > 0 && ahead(i - 1)) {
+    L.hl_sc[i][lane] = L.hl_sc[i - 1][lane];
     W.hl_tot[i][lane] = W.hl_tot[i - 1][lane];
-    W.hl_id[i][lane] = pi;
     W.hl_pos[i][lane] = W.hl_pos[i - 1][lane];
     --i;
   }
   L.hl_sc[i][lane] = sc;
   W.hl_tot[i][lane] = tot;
-  W.hl_id[i][lane] = id;
   W.hl_pos[i][lane] = pos;
   ++n;
 }
 
 // Reorder a lane's kept list by (total chi2, hit id) and keep at most cap entries.
 template <int KC>
-__device__ __forceinline__ void hl_sort_by_chi2(WarpSmem<KC>& W, int lane, int& n, int cap) {
+__device__ __forceinline__ void hl_sort_by_chi2(WarpSmem<KC>& W, const float4* __restrict__ rec, int lane, int& n,
+                                                int cap) {
   for (int i = 1; i < n; ++i) {
     const float c = W.hl_tot[i][lane];
-    const int id = W.hl_id[i][lane], pos = W.hl_pos[i][lane];
+    const int pos = W.hl_pos[i][lane];
     int j = i;
-    while (j > 0 && before(c, id, W.hl_tot[j - 1][lane], W.hl_id[j - 1][lane])) {
+    while (j > 0 && before(rec, c, pos, W.hl_tot[j - 1][lane], W.hl_pos[j - 1][lane])) {
       W.hl_tot[j][lane] = W.hl_tot[j - 1][lane];
-      W.hl_id[j][lane] = W.hl_id[j - 1][lane];
       W.hl_pos[j][lane] = W.hl_pos[j - 1][lane];
       --j;
     }
     W.hl_tot[j][lane] = c;
-    W.hl_id[j][lane] = id;
     W.hl_pos[j][lane] = pos;
   }
   if (n > cap) n = cap;
@@ -259,25 +257,24 @@ __device__ __forceinline__ float update_exact(const DevGeom& G, int si, Cand& c,
   return kalman_update(c.p, c.C, in, m.r0, m.r1);
 }
 
-// Insert (tot, id, pos) into lane's list sorted by (total chi2, hit id), capacity cap (holding n).
+// Insert (tot, pos) into lane's list sorted by (total chi2, hit id), capacity cap (holding n).
 template <int KC>
-__device__ __forceinline__ void hl_insert(WarpSmem<KC>& W, int lane, int& n, int cap, float tot, int id, int pos) {
+__device__ __forceinline__ void hl_insert(WarpSmem<KC>& W, const float4* __restrict__ rec, int lane, int& n, int cap,
+                                          float tot, int pos) {
   if (n == cap) {
-    if (!before(tot, id, W.hl_tot[cap - 1][lane], W.hl_id[cap - 1][lane])) return;
+    if (!before(rec, tot, pos, W.hl_tot[cap - 1][lane], W.hl_pos[cap - 1][lane])) return;
     n = cap - 1;
   }
   int i = n;
   while (i > 0) {
     const float pc = W.hl_tot[i - 1][lane];
-    const int pi = W.hl_id[i - 1][lane];
-    if (!before(tot, id, pc, pi)) break;
+    const int pp = W.hl_pos[i - 1][lane];
+    if (!before(rec, tot, pos, pc, pp)) break;
     W.hl_tot[i][lane] = pc;
-    W.hl_id[i][lane] = pi;
-    W.hl_pos[i][lane] = W.hl_pos[i - 1][lane];
+    W.hl_pos[i][lane] = pp;
     --i;
   }
   W.hl_tot[i][lane] = tot;
-  W.hl_id[i][lane] = id;
   W.hl_pos[i][lane] = pos;
   ++n;
 }
@@ -716,7 +713,7 @@ __global__ void __launch_bounds__(LEARNED ? kFindMaxBlockLearned : 256, 2) k_fin
             const bool real = j < total_sc;
             float x12 = 0.f, x13 = 0.f;
             if (real && t4 == 2) {
-              const float4 hr = __ldg(A.sorted_rec + W.u.pl.pos[k]);
+              const float4 hr = __ldg(A.sorted_rec + W.pl.pos[k]);
               float q0, q1;
               window_chi2(W.win_a[o], W.win_b[o], hr, q0, q1);
               x12 = (q0 / d12 - __ldg(wmlp + kMlpMean + 12)) / __ldg(wmlp + kMlpSd + 12);
@@ -742,21 +739,20 @@ __global__ void __launch_bounds__(LEARNED ? kFindMaxBlockLearned : 256, 2) k_fin
           __syncwarp();
           if ((needmask >> lane) & 1u)
             for (int k = start; k < start + my_cnt; ++k)
-              hl_insert_scored(W, WL, lane, hl_n, keep, WL.pl_sc[k], c.chi2 + W.u.pl.c2[k], W.u.pl.id[k],
-                               W.u.pl.c2[k] < cut ? W.u.pl.pos[k] : ~W.u.pl.pos[k]);
+              hl_insert_scored(W, WL, A.sorted_rec, lane, hl_n, keep, WL.pl_sc[k], c.chi2 + W.pl.c2[k],
+                               W.pl.c2[k] < cut ? W.pl.pos[k] : ~W.pl.pos[k]);
         }
         if (!need) {  // kept unconditionally (at most top_n of them)
           for (int k = start; k < start + my_cnt; ++k) {
-            W.hl_tot[hl_n][lane] = c.chi2 + W.u.pl.c2[k];
-            W.hl_id[hl_n][lane] = W.u.pl.id[k];
-            W.hl_pos[hl_n][lane] = W.u.pl.c2[k] < cut ? W.u.pl.pos[k] : ~W.u.pl.pos[k];
+            W.hl_tot[hl_n][lane] = c.chi2 + W.pl.c2[k];
+            W.hl_pos[hl_n][lane] = W.pl.c2[k] < cut ? W.pl.pos[k] : ~W.pl.pos[k];
             ++hl_n;
           }
         }
         scored = scored || (need && my_cnt > 0);
       } else {
         for (int k = start; k < start + my_cnt; ++k)
-          hl_insert(W, lane, hl_n, keep, c.chi2 + W.u.pl.c2[k], W.u.pl.id[k], W.u.pl.pos[k]);
+          hl_insert(W, A.sorted_rec, lane, hl_n, keep, c.chi2 + W.pl.c2[k], W.pl.pos[k]);
         npass += my_cnt;
       }
       my_cnt = 0;
@@ -823,13 +819,11 @@ __global__ void __launch_bounds__(LEARNED ? kFindMaxBlockLearned : 256, 2) k_fin
           }
           const int pos = o + adj;
           float c2v = __int_as_float(0x7f800000);
-          int hid = 0;
           bool inbox = false;
           if (q < total) {
             const float4 h = __ldg(A.sorted_rec + pos);
             float r0, r1;
             c2v = window_chi2(W.win_a[owner], W.win_b[owner], h, r0, r1);
-            hid = __float_as_int(h.w);
             // Window ranking buffers every hit of the box of the chi2 ellipse (a hit rejected by the
             // angular pre-test, c2v infinite, lies outside it).
             if (LEARNED && window_rank) {
@@ -848,10 +842,8 @@ __global__ void __launch_bounds__(LEARNED ? kFindMaxBlockLearned : 256, 2) k_fin
           }
           if (pass) {
             const int k = np + __popc(m & ((1u << lane) - 1u));
-            W.u.pl.c2[k] = c2v;
-            W.u.pl.id[k] = hid;
-            W.u.pl.pos[k] = pos;
-            if (LEARNED) W.u.pl.own[k] = owner;
+            W.pl.c2[k] = c2v;
+            W.pl.pos[k] = pos;
           }
           np += __popc(m);
         }
@@ -883,13 +875,12 @@ __global__ void __launch_bounds__(LEARNED ? kFindMaxBlockLearned : 256, 2) k_fin
       for (int k = 0; k < hl_n; ++k) {
         if (W.hl_pos[k][lane] < 0) continue;
         W.hl_tot[m][lane] = W.hl_tot[k][lane];
-        W.hl_id[m][lane] = W.hl_id[k][lane];
         W.hl_pos[m][lane] = W.hl_pos[k][lane];
         ++m;
       }
       hl_n = m;
     }
-    if (LEARNED && hl_n > 0) hl_sort_by_chi2(W, lane, hl_n, cap);
+    if (LEARNED && hl_n > 0) hl_sort_by_chi2(W, A.sorted_rec, lane, hl_n, cap);
     // Outcome of each propagated candidate; keep the prediction for its children.
     if (kind == 1) {
       kind = hl_n > 0 ? 0 : (c.nm < A.max_miss ? 1 : 2);
@@ -938,7 +929,6 @@ __global__ void __launch_bounds__(LEARNED ? kFindMaxBlockLearned : 256, 2) k_fin
       const unsigned long long gm = __shfl_sync(kFull, m, gbase);
       if (in_grp && mk != ~0ull && mk == gm) {
         W.tab_key[gbase + r] = mk;
-        W.tab_id[gbase + r] = kind == 0 ? W.hl_id[head][lane] : -1;
         W.tab_pos[gbase + r] = kind == 0 ? W.hl_pos[head][lane] : 0;
         ++head;
         mk = nk;
@@ -954,7 +944,6 @@ __global__ void __launch_bounds__(LEARNED ? kFindMaxBlockLearned : 256, 2) k_fin
         const int pk = static_cast<int>((mk >> 20) & 63ull);
         w_par = pk >> 2;
         w_kind = pk & 3;
-        w_id = W.tab_id[lane];
         w_pos = W.tab_pos[lane];
         w_nh = 63 - static_cast<int>(mk >> 58);
         w_c2 = __uint_as_float(static_cast<unsigned>((mk >> 26) & 0xffffffffull));
@@ -968,6 +957,7 @@ __global__ void __launch_bounds__(LEARNED ? kFindMaxBlockLearned : 256, 2) k_fin
       load_cand(W, gbase + w_par, nc);
       if (w_kind == 0) {
         const float4 h = __ldg(A.sorted_rec + w_pos);
+        w_id = __float_as_int(h.w);
         update_with(G, STEER ? nc.surf & 255 : nc.surf, nc, h);
         nc.chi2 = w_c2;
         nc.nh = w_nh;
