@@ -758,30 +758,32 @@ __global__ void __launch_bounds__(LEARNED ? kFindMaxBlockLearned : 256, 2) k_fin
       my_cnt = 0;
     };
     for (;;) {
-      int T = 0;
+      // The bounds of a run over whole phi sub-bins are two bin offsets, those of a limited run (one
+      // bin) a bin offset and two sub-bin counts; all loads of a pass are issued together.
+      int o0[kRows], o1[kRows], u0[kRows], u1[kRows];
 #pragma unroll
       for (int k = 0; k < kRows; ++k) {
-        int a = 0, b = 0;
+        o0[k] = o1[k] = u0[k] = u1[k] = 0;
         if (row < npb) {
           int pb = pb0 + row;
           if (pb >= nphi) pb -= nphi;
           const int slo = row == 0 ? sub_of(flo, pb) : 0;
           const int shi = row == npb - 1 ? sub_of(fhi, pb) : kPhiSub - 1;
-          if (slo == 0 && shi == kPhiSub - 1) {
-            a = __ldg(off + pb * n2 + zb0);
-            b = __ldg(off + pb * n2 + zb1 + 1);
-            ++row;
-          } else {
-            const int bb = pb * n2 + zrun;
-            const int s0 = __ldg(off + bb);
-            a = s0 + (slo > 0 ? __ldg(sub + bb * kPhiSub + slo - 1) : 0);
-            b = s0 + __ldg(sub + bb * kPhiSub + shi);
-            if (++zrun > zb1) {
-              zrun = zb0;
-              ++row;
-            }
-          }
+          const bool whole = slo == 0 && shi == kPhiSub - 1;
+          const int bb = pb * n2 + (whole ? zb0 : zrun);
+          o0[k] = __ldg(off + bb);
+          o1[k] = __ldg(off + (whole ? pb * n2 + zb1 + 1 : bb));
+          if (slo > 0) u0[k] = __ldg(sub + bb * kPhiSub + slo - 1);
+          if (!whole) u1[k] = __ldg(sub + bb * kPhiSub + shi);
+          const bool next = whole || zrun >= zb1;
+          zrun = next ? zb0 : zrun + 1;
+          row += next;
         }
+      }
+      int T = 0;
+#pragma unroll
+      for (int k = 0; k < kRows; ++k) {
+        const int a = o0[k] + u0[k], b = o1[k] + u1[k];
         W.rows[k][lane] = make_int2(T + (b - a), a - T);
         T += b - a;
       }
