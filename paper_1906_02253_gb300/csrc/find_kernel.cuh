@@ -50,12 +50,14 @@ struct WarpSmem {
   int2 rows[kRows][32];    // runs: (end of the run in the lane's flattened window, position - start)
   float hl_tot[KC][32];    // per lane: best passing hits, sorted by (total chi2, hit id), and their
   int hl_pos[KC][32];      // positions in the index (the record there holds the id)
-  unsigned long long tab_key[32];  // winner table of each group, by rank
-  int tab_pos[32];
-  struct {
-    float c2[kPList];
-    int pos[kPList];
-  } pl;  // buffered passing pairs (scan)
+  unsigned long long win[32];  // keys of each group's best children, by rank
+  union {
+    struct {
+      float c2[kPList];
+      int pos[kPList];
+    } pl;                                      // buffered passing pairs (scan)
+    __align__(16) unsigned long long key[64];  // keys of the children being ranked, 2 KC per group (selection)
+  } u;
 };
 
 // Learned instances of up to 4 slots hold the network's weight fragments in shared memory, after
@@ -441,7 +443,8 @@ __device__ __noinline__ void write_track(const WarpSmem<KC>& W, const int* trace
   status_out[seed] = 0;
 }
 
-// Packed ranking key: (63 - hits) << 58 | chi2 bits << 26 | (parent slot << 2 | kind) << 20.
+// Packed ranking key: (63 - hits) << 58 | chi2 bits << 26 | (parent slot << 2 | kind) << 20 (| place
+// in the parent's list, which is by chi2 and hit id).
 // For chi2 >= 0 its IEEE bits order like its value (a rounding-negative chi2 ranks as 0); the hit
 // id breaks remaining ties.
 __device__ __forceinline__ unsigned long long pack_key(int nh, float c2, int pk) {
@@ -713,7 +716,7 @@ __global__ void __launch_bounds__(LEARNED ? kFindMaxBlockLearned : 256, 2) k_fin
             const bool real = j < total_sc;
             float x12 = 0.f, x13 = 0.f;
             if (real && t4 == 2) {
-              const float4 hr = __ldg(A.sorted_rec + W.pl.pos[k]);
+              const float4 hr = __ldg(A.sorted_rec + W.u.pl.pos[k]);
               float q0, q1;
               window_chi2(W.win_a[o], W.win_b[o], hr, q0, q1);
               x12 = (q0 / d12 - __ldg(wmlp + kMlpMean + 12)) / __ldg(wmlp + kMlpSd + 12);
@@ -739,20 +742,20 @@ __global__ void __launch_bounds__(LEARNED ? kFindMaxBlockLearned : 256, 2) k_fin
           __syncwarp();
           if ((needmask >> lane) & 1u)
             for (int k = start; k < start + my_cnt; ++k)
-              hl_insert_scored(W, WL, A.sorted_rec, lane, hl_n, keep, WL.pl_sc[k], c.chi2 + W.pl.c2[k],
-                               W.pl.c2[k] < cut ? W.pl.pos[k] : ~W.pl.pos[k]);
+              hl_insert_scored(W, WL, A.sorted_rec, lane, hl_n, keep, WL.pl_sc[k], c.chi2 + W.u.pl.c2[k],
+                               W.u.pl.c2[k] < cut ? W.u.pl.pos[k] : ~W.u.pl.pos[k]);
         }
         if (!need) {  // kept unconditionally (at most top_n of them)
           for (int k = start; k < start + my_cnt; ++k) {
-            W.hl_tot[hl_n][lane] = c.chi2 + W.pl.c2[k];
-            W.hl_pos[hl_n][lane] = W.pl.c2[k] < cut ? W.pl.pos[k] : ~W.pl.pos[k];
+            W.hl_tot[hl_n][lane] = c.chi2 + W.u.pl.c2[k];
+            W.hl_pos[hl_n][lane] = W.u.pl.c2[k] < cut ? W.u.pl.pos[k] : ~W.u.pl.pos[k];
             ++hl_n;
           }
         }
         scored = scored || (need && my_cnt > 0);
       } else {
         for (int k = start; k < start + my_cnt; ++k)
-          hl_insert(W, A.sorted_rec, lane, hl_n, keep, c.chi2 + W.pl.c2[k], W.pl.pos[k]);
+          hl_insert(W, A.sorted_rec, lane, hl_n, keep, c.chi2 + W.u.pl.c2[k], W.u.pl.pos[k]);
         npass += my_cnt;
       }
       my_cnt = 0;
@@ -844,8 +847,8 @@ __global__ void __launch_bounds__(LEARNED ? kFindMaxBlockLearned : 256, 2) k_fin
           }
           if (pass) {
             const int k = np + __popc(m & ((1u << lane) - 1u));
-            W.pl.c2[k] = c2v;
-            W.pl.pos[k] = pos;
+            W.u.pl.c2[k] = c2v;
+            W.u.pl.pos[k] = pos;
           }
           np += __popc(m);
         }
@@ -895,60 +898,125 @@ __global__ void __launch_bounds__(LEARNED ? kFindMaxBlockLearned : 256, 2) k_fin
 
     // ---- 3. selection of the k_max best children of each seed -----------------------------
     // Each lane offers its children in ranking order (hit children by total chi2, or one miss or
-    // carried child) as a list whose head key is in a register; k_max rounds of a tournament
-    // over the group's heads (a segmented minimum by shuffles) give the seed's children in rank
-    // order, and the child of rank j goes to the group's slot j. Keys of different lanes differ
-    // (they carry the slot), so the order is the same total order as comparing all children.
+    // carried child). Keys of different children differ (they carry the parent's slot and the place
+    // in its list), so their order is total, and the child of rank j goes to the group's slot j. Two
+    // ways to rank them, the same result:
+    //  - the plain instances without options count: the group's children are numbered lane by lane,
+    //    their keys gathered in shared memory, 2 KC at a time, and each lane counts the smaller
+    //    keys of one or two of them; more children than 2 KC: the KC best meet the next KC;
+    //  - the others run a tournament: each list's head key is in a register; up to k_max rounds of a
+    //    segmented minimum by shuffles.
+    // Counting shortens the step by 5% at 6 slots (100 barrel events, finder 10.2 against 9.6 ms)
+    // and 2% on barrel + disks; in the larger learned and option instances it is 2-4% slower.
     // In a detecting pass a seed whose children outnumber the slots overflows: its group takes no
     // part in the selection and the seed goes to the second pass (its children all fit otherwise,
     // and keeping them all is what the full capacity does).
+    constexpr bool RANK = !LEARNED && FEAT == 0;
     int nch = (on && kind != 3) ? (kind == 0 ? (detect && !LEARNED ? npass : hl_n) : 1) : 0;
-    // Rounds: the most children any group of the warp has, up to k_max.
-    int tot = nch;
-#pragma unroll
-    for (int off = 1; off < KC; off <<= 1) {
-      const int v = __shfl_down_sync(kFull, tot, off);
-      if (slot + off < KC) tot += v;
-    }
-    const bool ovf = detect && __shfl_sync(kFull, tot, gbase) > KC;
-    if (ovf) nch = 0;
-    const int rounds =
-        min(cap, static_cast<int>(__reduce_max_sync(kFull, in_grp && slot == 0 && !ovf ? tot : 0)));
-    unsigned long long mk = ~0ull, nk = ~0ull;  // this lane's head key and the one after it
-    if (nch > 0) mk = kind == 0 ? pack_key(c.nh + 1, W.hl_tot[0][lane], slot << 2) : pack_key(c.nh, c.chi2, (slot << 2) | kind);
-    if (nch > 1) nk = pack_key(c.nh + 1, W.hl_tot[1][lane], slot << 2);
-    int head = 0;
-    W.tab_key[lane] = ~0ull;
-    __syncwarp();
-#pragma unroll 1
-    for (int r = 0; r < rounds; ++r) {
-      unsigned long long m = mk;
+    auto child_key = [&](int h) {
+      return kind == 0 ? pack_key(c.nh + 1, W.hl_tot[h][lane], slot << 2) | static_cast<unsigned>(h)
+                       : pack_key(c.nh, c.chi2, (slot << 2) | kind);
+    };
+    bool ovf;
+    if constexpr (RANK) {
+      int cincl = nch;
 #pragma unroll
       for (int off = 1; off < KC; off <<= 1) {
-        const unsigned long long v = __shfl_down_sync(kFull, m, off);
-        if (slot + off < KC) m = v < m ? v : m;
+        const int v = __shfl_up_sync(kFull, cincl, off);
+        if (slot >= off) cincl += v;
       }
-      const unsigned long long gm = __shfl_sync(kFull, m, gbase);
-      if (in_grp && mk != ~0ull && mk == gm) {
-        W.tab_key[gbase + r] = mk;
-        W.tab_pos[gbase + r] = kind == 0 ? W.hl_pos[head][lane] : 0;
-        ++head;
-        mk = nk;
-        nk = head + 1 < nch ? pack_key(c.nh + 1, W.hl_tot[head + 1][lane], slot << 2) : ~0ull;
+      const int all = __shfl_sync(kFull, cincl, in_grp ? gbase + KC - 1 : lane), tot = in_grp ? all : 0;
+      ovf = detect && tot > KC;
+      const int first = cincl - nch;  // number of this lane's first child
+      if (ovf) nch = 0;
+      const int most = static_cast<int>(__reduce_max_sync(kFull, ovf ? 0 : tot));
+      unsigned long long* const kb = W.u.key + (in_grp ? grp * 2 * KC : 0);
+      auto gather = [&](int c0, int c1, int at) {  // children numbered [c0, c1) to kb[at ...]
+        for (int h = max(0, c0 - first); h < min(nch, c1 - first); ++h) kb[at + first + h - c0] = child_key(h);
+      };
+      if (in_grp) kb[slot] = kb[KC + slot] = ~0ull;
+      __syncwarp();
+      gather(0, 2 * KC, 0);
+      for (int c0 = 2 * KC;; c0 += KC) {
+        W.win[lane] = ~0ull;
+        __syncwarp();
+        if (most <= KC) {  // one child a lane at most (warp-uniform)
+          if (in_grp) {
+            const unsigned long long ka = kb[slot];
+            int ra = 0;
+#pragma unroll
+            for (int j = 0; j < (KC + 1) / 2; ++j) {
+              const ulonglong2 v = reinterpret_cast<const ulonglong2*>(kb)[j];
+              ra += (v.x < ka) + (v.y < ka);
+            }
+            if (ka != ~0ull && ra < cap) W.win[gbase + ra] = ka;
+          }
+        } else if (in_grp) {
+          const unsigned long long ka = kb[slot], kz = kb[KC + slot];
+          int ra = 0, rz = 0;
+#pragma unroll
+          for (int j = 0; j < KC; ++j) {
+            const ulonglong2 v = reinterpret_cast<const ulonglong2*>(kb)[j];
+            ra += (v.x < ka) + (v.y < ka);
+            rz += (v.x < kz) + (v.y < kz);
+          }
+          if (ka != ~0ull && ra < cap) W.win[gbase + ra] = ka;
+          if (kz != ~0ull && rz < cap) W.win[gbase + rz] = kz;
+        }
+        __syncwarp();
+        if (c0 >= most) break;
+        if (in_grp) {
+          kb[slot] = W.win[lane];
+          kb[KC + slot] = ~0ull;
+        }
+        __syncwarp();
+        gather(c0, c0 + KC, KC);
       }
+    } else {
+      int tot = nch;
+#pragma unroll
+      for (int off = 1; off < KC; off <<= 1) {
+        const int v = __shfl_down_sync(kFull, tot, off);
+        if (slot + off < KC) tot += v;
+      }
+      ovf = detect && __shfl_sync(kFull, tot, gbase) > KC;
+      if (ovf) nch = 0;
+      const int rounds =
+          min(cap, static_cast<int>(__reduce_max_sync(kFull, in_grp && slot == 0 && !ovf ? tot : 0)));
+      unsigned long long mk = nch > 0 ? child_key(0) : ~0ull;  // this lane's head key and the one after it
+      unsigned long long nk = nch > 1 ? child_key(1) : ~0ull;
+      int head = 0;
+      W.win[lane] = ~0ull;
+      __syncwarp();
+#pragma unroll 1
+      for (int r = 0; r < rounds; ++r) {
+        unsigned long long m = mk;
+#pragma unroll
+        for (int off = 1; off < KC; off <<= 1) {
+          const unsigned long long v = __shfl_down_sync(kFull, m, off);
+          if (slot + off < KC) m = v < m ? v : m;
+        }
+        const unsigned long long gm = __shfl_sync(kFull, m, gbase);
+        if (in_grp && mk != ~0ull && mk == gm) {
+          W.win[gbase + r] = mk;
+          ++head;
+          mk = nk;
+          nk = head + 1 < nch ? child_key(head + 1) : ~0ull;
+        }
+      }
+      __syncwarp();
     }
-    __syncwarp();
     int w_par = 0, w_kind = 3, w_id = -1, w_pos = 0, w_nh = 0;
     float w_c2 = 0.f;
     if (on) {
-      const unsigned long long mk = W.tab_key[lane];
+      const unsigned long long mk = W.win[lane];
       if (mk != ~0ull) {
         const int pk = static_cast<int>((mk >> 20) & 63ull);
         w_par = pk >> 2;
         w_kind = pk & 3;
-        w_pos = W.tab_pos[lane];
         w_nh = 63 - static_cast<int>(mk >> 58);
         w_c2 = __uint_as_float(static_cast<unsigned>((mk >> 26) & 0xffffffffull));
+        if (w_kind == 0) w_pos = W.hl_pos[static_cast<int>(mk & 0xfffffull)][gbase + w_par];
       }
     }
 
