@@ -358,6 +358,7 @@ static int prepare_find(const KfGeometry* geom, const KfHitIndex* index, const f
   A->score_margin = params->mlp ? params->score_margin : 0.f;
   A->window_rank = params->mlp ? params->window_ranking : 0;
   A->seed_keep = params->seed_keep;
+  A->class_count = nullptr;
   return KF_OK;
 }
 
@@ -377,8 +378,8 @@ int kf_find_tracks(const KfGeometry* geom, const KfHitIndex* index, const float*
   const int rc = prepare_find(geom, index, hits, hit_surface, seed_hits, seed_event, n_seeds, params, hits_out,
                               nhits_out, chi2_out, state_out, cov_out, status_out, -1, &G, &M, &plan, &A, &empty);
   if (rc != KF_OK || empty) return rc;
-  if (!workspace || workspace_bytes < plan.ws_bytes || (reinterpret_cast<size_t>(workspace) & 255)) return KF_ERR_ARG;
-  return launch_find(G, M, A, plan, workspace, reinterpret_cast<cudaStream_t>(stream));
+  if (!workspace || workspace_bytes < plan.need_bytes || (reinterpret_cast<size_t>(workspace) & 255)) return KF_ERR_ARG;
+  return launch_find(G, M, A, plan, workspace, workspace_bytes, reinterpret_cast<cudaStream_t>(stream));
 }
 
 int kf_seed_states(const KfGeometry* geom, const float* hits, const int* hit_surface, const int* seed_hits,
@@ -450,12 +451,13 @@ int kf_find_tracks_static(const KfGeometry* geom, const KfHitIndex* index, const
   int rc = prepare_find(geom, index, hits, hit_surface, seed_hits, seed_event, n_seeds, params, hits_out, nhits_out,
                         chi2_out, state_out, cov_out, status_out, KF_STATIC_MAX_SEEDS, &G, &M, &plan, &A, &empty);
   if (rc != KF_OK) return rc;
-  if (plan.ws_bytes > KF_STATIC_SCRATCH_BYTES) return KF_ERR_CAPACITY;
+  if (plan.need_bytes > KF_STATIC_SCRATCH_BYTES) return KF_ERR_CAPACITY;
   if (empty) return KF_OK;
   void* scratch = nullptr;
   rc = static_scratch(&scratch);
   if (rc != KF_OK) return rc;
-  return launch_find(G, M, A, plan, scratch, reinterpret_cast<cudaStream_t>(stream));
+  // (need_bytes: seeds in index order at every size, not ordered where a smaller call leaves room)
+  return launch_find(G, M, A, plan, scratch, plan.need_bytes, reinterpret_cast<cudaStream_t>(stream));
 }
 
 // ---- autotuners: time each configuration with CUDA events on the caller's stream ---------------

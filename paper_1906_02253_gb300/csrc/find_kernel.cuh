@@ -404,43 +404,55 @@ __device__ __forceinline__ int next_surface(const DevGeom& G, const float* p, in
   return sel;
 }
 
-// Words per seed of the seed states k_seed_states writes (p[6], C[21], chi2).
+// Words per seed of the finder's seed records (p[6], C[21], chi2; chi2 < 0: failed): 112 bytes, the first
+// seven 16-byte words of a candidate record.
 constexpr int kSeedWords = 28;
 
-// A fresh seed's state (fitted by k_seed_states, structure of arrays with stride n) into the
-// candidate record of `lane`; false for a failed seed. Out of line: once per seed.
+// A fresh seed's record into the candidate record of the group's first slot, its 16-byte words
+// spread over the group's lanes; false for a failed seed.
 template <int KC>
-__device__ __noinline__ bool load_seed(WarpSmem<KC>& W, int lane, const float* in, int surf_word, int n) {
-  const float chi2 = in[static_cast<size_t>(27) * n];
-  if (!(chi2 >= 0.f)) return false;
-  for (int i = 0; i < 27; ++i) cand_word(W, i, lane) = in[static_cast<size_t>(i) * n];
-  cand_word(W, 27, lane) = chi2;
-  cand_word(W, 28, lane) = __int_as_float(3);  // hits
-  cand_word(W, 29, lane) = __int_as_float(0);  // misses
-  cand_word(W, 30, lane) = __int_as_float(0);  // stopped
-  cand_word(W, 31, lane) = __int_as_float(surf_word);
+__device__ __forceinline__ bool load_seed(WarpSmem<KC>& W, int gbase, int slot, const float* rec, int surf_word) {
+  const float4* r4 = reinterpret_cast<const float4*>(rec);
+  if (!(__ldg(rec + 27) >= 0.f)) return false;
+#pragma unroll
+  for (int i = 0; i < kSeedWords / 4; i += KC)
+    if (i + slot < kSeedWords / 4) W.cand[i + slot][gbase] = __ldg(r4 + i + slot);
+  if (slot == 0)  // 3 hits, no miss, not stopped
+    W.cand[kSeedWords / 4][gbase] =
+        make_float4(__int_as_float(3), __int_as_float(0), __int_as_float(0), __int_as_float(surf_word));
   return true;
+}
+// The same out of line, for the small plain instances and the steering ones: inlined there it makes
+// the compiler round one of the step's sums differently from the other instances, and an adaptive
+// capacity's two instances have to agree bit for bit (a test holds them to it). Elsewhere inlining
+// is faster (learned finding by 6%).
+template <int KC>
+__device__ __noinline__ bool load_seed_call(WarpSmem<KC>& W, int gbase, int slot, const float* rec, int surf_word) {
+  return load_seed(W, gbase, slot, rec, surf_word);
 }
 
 // Output of a finished seed: the best candidate (slot 0 of the group at gbase) and its hit list,
-// backtracked through the per-step trace of (parent slot, hit id + 1). Out of line: once per seed.
+// backtracked through the per-step trace of (parent slot, hit id + 1); the state and covariance
+// words are spread over the group's lanes. Out of line: once per seed.
 template <int KC>
-__device__ __noinline__ void write_track(const WarpSmem<KC>& W, const int* trace, int gbase, int step, int seed, int n,
-                                         int lmax, const int* seed_hits, int* hits_out, int* nhits_out,
+__device__ __noinline__ void write_track(const WarpSmem<KC>& W, const int* trace, int gbase, int slot, int step,
+                                         int seed, int n, int lmax, const int* seed_hits, int* hits_out, int* nhits_out,
                                          float* chi2_out, float* state_out, float* cov_out, int* status_out) {
+#pragma unroll 1
+  for (int w = slot; w < 27; w += KC)
+    (w < 6 ? state_out + static_cast<size_t>(w) * n : cov_out + static_cast<size_t>(w - 6) * n)[seed] = cand_word(W, w, gbase);
+  for (int k = 3 + step + slot; k < lmax; k += KC) hits_out[static_cast<size_t>(k) * n + seed] = -1;
+  for (int k = slot; k < 3; k += KC) hits_out[static_cast<size_t>(k) * n + seed] = seed_hits[static_cast<size_t>(k) * n + seed];
+  if (slot != 0) return;
+  nhits_out[seed] = __float_as_int(cand_word(W, 28, gbase));
+  chi2_out[seed] = cand_word(W, 27, gbase);
+  status_out[seed] = 0;
   int sl = 0;
   for (int st = step - 1; st >= 0; --st) {
     const int e = trace[st * 32 + gbase + sl];
     hits_out[static_cast<size_t>(3 + st) * n + seed] = (e & ((1 << kHitBits) - 1)) - 1;
     sl = e >> kHitBits;
   }
-  for (int k = 3 + step; k < lmax; ++k) hits_out[static_cast<size_t>(k) * n + seed] = -1;
-  for (int k = 0; k < 3; ++k) hits_out[static_cast<size_t>(k) * n + seed] = seed_hits[static_cast<size_t>(k) * n + seed];
-  nhits_out[seed] = __float_as_int(cand_word(W, 28, gbase));
-  chi2_out[seed] = cand_word(W, 27, gbase);
-  for (int i = 0; i < 6; ++i) state_out[static_cast<size_t>(i) * n + seed] = cand_word(W, i, gbase);
-  for (int i = 0; i < 21; ++i) cov_out[static_cast<size_t>(i) * n + seed] = cand_word(W, 6 + i, gbase);
-  status_out[seed] = 0;
 }
 
 // Packed ranking key: (63 - hits) << 58 | chi2 bits << 26 | (parent slot << 2 | kind) << 20 (| place
@@ -549,8 +561,7 @@ __global__ void __launch_bounds__(LEARNED ? kFindMaxBlockLearned : 256, 2) k_fin
     if (!__syncthreads_or(seed >= 0)) break;
 
     // ---- a fresh group loads its seed state into slot 0 ------------------------------------
-    int failed = 0;
-    if (fresh && slot == 0) {
+    if (fresh) {
       // Candidate surface word: (position in the region's list + 1) << 8 | surface.
       const int s3 = A.seed_surf[seed];
       int pos = -1;
@@ -558,15 +569,14 @@ __global__ void __launch_bounds__(LEARNED ? kFindMaxBlockLearned : 256, 2) k_fin
         region = seed_region(G, s3, A.hits[A.seed_hits[static_cast<size_t>(2) * n + seed]]);
         pos = G.steer_pos[region][s3];
       }
-      valid = load_seed(W, lane, A.seed_state + seed, STEER ? ((pos + 1) << 8) | (s3 & 255) : s3, n);
-      failed = !valid;  // a failed seed's outputs were written by the seed-state kernel
+      const float* rec = A.seed_state + static_cast<size_t>(seed) * kSeedWords;
+      const int surf_word = STEER ? ((pos + 1) << 8) | (s3 & 255) : s3;
+      if constexpr (!LEARNED && (KC <= 4 || FEAT == kFeatSteer)) valid = load_seed_call(W, gbase, slot, rec, surf_word);
+      else valid = load_seed(W, gbase, slot, rec, surf_word);
+      if (!valid) seed = -1;  // a failed seed's outputs were written by the seed-state kernel
+      valid = valid && slot == 0;
     }
-    failed = __shfl_sync(kFull, failed, gbase);
-    if (STEER) region = __shfl_sync(kFull, region, gbase);
-    if (fresh && failed) {
-      seed = -1;
-      valid = false;
-    }
+    __syncwarp();
     const bool on = seed >= 0;
 
     // ---- 1. propagation and window set-up -------------------------------------------------
@@ -1049,13 +1059,14 @@ __global__ void __launch_bounds__(LEARNED ? kFindMaxBlockLearned : 256, 2) k_fin
     if (on) ++step;
     const unsigned live = __ballot_sync(kFull, on && won && !nc.stopped);
     const bool done = on && (((live & gmask) == 0u) || step >= max_steps);
-    if (done && slot == 0) {
-      if (ovf) {
+    if (done) {
+      if (!ovf) {
+        write_track(W, trace, gbase, slot, step, seed, n, A.lmax, A.seed_hits, A.hits_out, A.nhits_out, A.chi2_out,
+                    A.state_out, A.cov_out, A.status_out);
+      } else if (slot == 0) {
         const int at = atomicAdd(A.ovf_count, 1);
         if (at < n) A.ovf_list[at] = seed;  // the list holds n entries (each seed appends once)
-      } else
-        write_track(W, trace, gbase, step, seed, n, A.lmax, A.seed_hits, A.hits_out, A.nhits_out, A.chi2_out,
-                    A.state_out, A.cov_out, A.status_out);
+      }
     }
     __syncwarp();
     if (done) {

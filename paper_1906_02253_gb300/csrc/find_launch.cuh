@@ -38,10 +38,12 @@ struct FindArgs {
   int* counter;
   float* seed_state;  // [28][n_seeds]: p[6], C[21], chi2 (< 0: failed seed)
   int* seed_surf;     // [n_seeds]: surface of the third seed hit
+  int* class_count;   // seeds of each direction class (the seed-state kernel counts them), or null
   // Adaptive capacity (plain finding): a first pass at a smaller capacity (detect = 1) finishes the
   // seeds whose children never outnumber its slots, which then have exactly the results of the
   // full capacity, and lists the others in ovf_list (*ovf_count of them) without writing their
-  // outputs; the second pass takes its seeds from that list (seed_list, *seed_list_count).
+  // outputs; the second pass takes its seeds from that list (seed_list, *seed_list_count). The
+  // first or only pass takes its seeds from the list ordered by direction, or in index order (null).
   int detect;
   int* ovf_list;
   int* ovf_count;
@@ -57,6 +59,7 @@ struct FindPlan {
   int feat;  // options compiled into the instance: 1 steering, 2 material map and energy loss, 4 field
   size_t smem;
   size_t off_state, off_surf, off_mlp, ws_bytes;
+  size_t need_bytes, off_order;  // workspace without the seed order's list, and the list's place
   // Adaptive capacity: the first pass's capacity (0 = a single pass), launch and shared memory,
   // and the overflow list's place in the workspace.
   int kc1, block1, grid1;
@@ -69,7 +72,8 @@ int plan_find(int n_seeds, const KfFindParams* p, int sms, int features, FindPla
 inline int find_features(const DevGeom& G, const DevMat& M) {
   return (G.steer != 0 ? 1 : 0) | ((M.map_on != 0 || M.eloss > 0.f) ? 2 : 0) | (G.field_on != 0 ? 4 : 0);
 }
-int launch_find(const DevGeom& G, const DevMat& M, FindArgs& A, const FindPlan& plan, void* ws, cudaStream_t stream);
+int launch_find(const DevGeom& G, const DevMat& M, FindArgs& A, const FindPlan& plan, void* ws, size_t ws_bytes,
+                cudaStream_t stream);
 // The seed-state kernel alone (A.hits_out null: failed seeds get chi2 = -1 only).
 int launch_seed_states(const DevGeom& G, const DevMat& M, const FindArgs& A, cudaStream_t stream);
 // Device address of the library's fixed finder scratch on the current device (looked up on the

@@ -1,0 +1,87 @@
+"""Finding with the seeds taken by direction (geometries with disks, a workspace of the full size) gives
+bit for bit what it gives with the seeds in index order (a workspace without the order's 4 bytes per
+seed), at the edges of the ordering kernel's blocks, with failed and removed seeds, in one pass and
+two, plain, learned and with options."""
+import ctypes
+import os
+
+import numpy as np
+import pytest
+import torch
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def kf():
+    import __graft_entry__ as ge
+    ge.build_library()
+    import paper_1906_02253_gb300 as k
+    k.load_library()
+    return k
+
+
+@pytest.fixture(scope="module")
+def batch(kf):
+    wl = synth.workload("field", n_events=2, tracks_lo=2300, tracks_hi=2300, seed=17)
+    b = synth.generate(wl)
+    return wl, kf.to_device_event_batch(b)
+
+
+def _up(v):
+    return (v + 255) // 256 * 256
+
+
+@pytest.mark.parametrize("n", [1, 2, 127, 128, 129, 2047, 2048, 2049, 4600])
+@pytest.mark.parametrize("option", ["plain", "two_passes", "learned", "field"])
+def test_order_changes_no_result(kf, batch, n, option):
+    wl, dev = batch
+    from dataclasses import replace
+    g = kf.Geometry(wl if option == "field" else replace(wl, field_z2=0.0, field_r2=0.0))
+    ix = kf.build_hit_index(g, dev["hits"], dev["slab_offsets"], 2, dev["max_slab_hits"])
+    some = torch.linspace(0, dev["seed_hits"].shape[1] - 1, n).long().cuda()
+    seeds, event = dev["seed_hits"][:, some].contiguous(), dev["seed_event"][some].contiguous()
+    keep = torch.ones(n, dtype=torch.int32, device="cuda")
+    if n > 10:
+        seeds[1, 3] = -1          # failed: no such hit
+        seeds[:, 5] = seeds[0, 5]  # failed: one hit three times
+        event[7] = 9              # failed: no such event
+        keep[::6] = 0             # removed by cleaning
+    net = None
+    if option == "learned":
+        z = np.load(os.path.join(os.path.dirname(kf.__file__), "data", "mlp_hi_occ.npz"))
+        net = kf.mlp_buffer(z["weights"], z["mean"], z["sd"])
+    prm = kf.find_params(wl.chi2_cut, wl.k_max, wl.max_miss, wl.lmax, seed_keep=keep, mlp=net, top_n=2 if net is not None else 0,
+                         score_margin=0.7 if net is not None else 0.0, adaptive_capacity=2 if option == "two_passes" else 0)
+    full = kf.find_workspace_size(n, prm)
+    room = torch.empty(full, dtype=torch.uint8, device="cuda")
+    P = lambda t: ctypes.c_void_p(t.data_ptr())  # noqa: E731
+    outs = []
+    for size in (full, full - _up(4 * n)):
+        out = dict(hits=torch.full((wl.lmax, n), -7, dtype=torch.int32, device="cuda"))
+        for k in ("nhits", "status"):
+            out[k] = torch.full((n,), -7, dtype=torch.int32, device="cuda")
+        out["chi2"] = torch.full((n,), -7.0, device="cuda")
+        out["state"], out["cov"] = torch.full((6, n), -7.0, device="cuda"), torch.full((21, n), -7.0, device="cuda")
+        rc = kf.load_library().kf_find_tracks(
+            g.ref, ctypes.byref(ix.c), P(dev["hits"]), P(dev["hit_surface"]), P(seeds), P(event), n, ctypes.byref(prm),
+            P(out["hits"]), P(out["nhits"]), P(out["chi2"]), P(out["state"]), P(out["cov"]), P(out["status"]), P(room), size,
+            ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+        assert rc == kf.KF_OK
+        outs.append({k: v.clone() for k, v in out.items()})
+    a, b = outs
+    for k in a:
+        assert torch.equal(a[k].view(torch.int32), b[k].view(torch.int32)), k
+    want = torch.where(keep == 0, 2, 0)
+    if n > 10:
+        for i in (3, 5, 7):
+            want[i] = 1 if keep[i] else 2
+    assert torch.equal(a["status"], want.to(torch.int32))
+    # a smaller one is refused
+    rc = kf.load_library().kf_find_tracks(
+        g.ref, ctypes.byref(ix.c), P(dev["hits"]), P(dev["hit_surface"]), P(seeds), P(event), n, ctypes.byref(prm), P(out["hits"]),
+        P(out["nhits"]), P(out["chi2"]), P(out["state"]), P(out["cov"]), P(out["status"]), P(room), full - _up(4 * n) - 256,
+        ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+    assert rc == kf.KF_ERR_ARG
