@@ -8,6 +8,7 @@
 #include "../../include/kfgb.h"
 #include "kf_math.cuh"
 #include "mlp.cuh"
+#include "pdl.cuh"
 
 namespace kfgb {
 
@@ -251,8 +252,8 @@ int kf_build_hit_index(const KfGeometry* geom, const float* hits, const int* sla
     smem_set[fine][dev] = static_cast<int>(smem);
   }
   auto launch = [&](auto kernel) {
-    kernel<<<n_slabs, 1024, smem, reinterpret_cast<cudaStream_t>(stream)>>>(
-        G, reinterpret_cast<const float2*>(hits), slab_offsets, n_slabs, cap, index->bin_off,
+    launch_pdl(
+        kernel, n_slabs, 1024, smem, reinterpret_cast<cudaStream_t>(stream), G, reinterpret_cast<const float2*>(hits), slab_offsets, n_slabs, cap, index->bin_off,
         reinterpret_cast<float2*>(index->sorted_hits), index->sorted_ids, reinterpret_cast<float4*>(index->sorted_rec),
         reinterpret_cast<uint4*>(index->sub_off), d_status);
   };
@@ -287,8 +288,8 @@ int kf_fit_tracks(const KfGeometry* geom, const float* hits, const int* hit_surf
   }
   const long long want = (static_cast<long long>(n_tracks) + block_threads - 1) / block_threads;
   const int grid = static_cast<int>(std::min<long long>(want, static_cast<long long>(sm_count()) * occ));
-  k_fit_tracks<<<grid, block_threads, 0, reinterpret_cast<cudaStream_t>(stream)>>>(
-      G, M, reinterpret_cast<const float2*>(hits), hit_surface, track_hits, n_tracks, lmax, state_out, cov_out, chi2_out,
+  launch_pdl(
+      k_fit_tracks, grid, block_threads, 0, reinterpret_cast<cudaStream_t>(stream), G, M, reinterpret_cast<const float2*>(hits), hit_surface, track_hits, n_tracks, lmax, state_out, cov_out, chi2_out,
       ndof_out, status_out);
   return launch_status();
 }

@@ -32,6 +32,7 @@ template <bool FIND>
 __global__ void __launch_bounds__(128) k_seed_states(DevGeom G, const __grid_constant__ DevMat M, FindArgs A) {
   const int seed = blockIdx.x * blockDim.x + threadIdx.x;
   const int n = A.n_seeds;
+  if (FIND && !A.class_count && seed < 3) A.counter[seed] = 0;  // the finder's work counters (else cleared with the classes')
   const bool in = seed < n;
   int ids[3] = {-1, -1, -1}, ev = -1;
   bool removed = false;
@@ -386,7 +387,8 @@ int launch_find(const DevGeom& G, const DevMat& M, FindArgs& A, const FindPlan& 
   constexpr int kCounters = 56;
   static_assert(8 + kClasses <= 32 && 32 + kClasses <= kCounters && kCounters * sizeof(int) <= 256, "counter area");
   const bool ordered = G.n_dpos + G.n_dneg > 0 && ws_bytes >= plan.ws_bytes;
-  if (cudaMemsetAsync(A.counter, 0, (ordered ? kCounters : 3) * sizeof(int), stream) != cudaSuccess) return KF_ERR_CUDA;
+  // The classes count from zero in the seed-state kernel, which else clears the queues itself.
+  if (ordered && cudaMemsetAsync(A.counter, 0, kCounters * sizeof(int), stream) != cudaSuccess) return KF_ERR_CUDA;
   A.detect = 0;
   A.ovf_list = A.ovf_count = nullptr;
   A.seed_list = A.seed_list_count = nullptr;

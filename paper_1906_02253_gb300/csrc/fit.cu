@@ -3,6 +3,7 @@
 // tracks of all events; the state (6) and the packed covariance (21) stay in registers through
 // all surfaces; track hit ids are read as structure-of-arrays (coalesced), hits gathered by id.
 #include "kf_math.cuh"
+#include "pdl.cuh"
 
 namespace kfgb {
 
@@ -13,6 +14,7 @@ __global__ void __launch_bounds__(256) k_fit_tracks(DevGeom G, const __grid_cons
                                                     float* __restrict__ state_out, float* __restrict__ cov_out,
                                                     float* __restrict__ chi2_out, int* __restrict__ ndof_out,
                                                     int* __restrict__ status_out) {
+  pdl_begin();
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n_tracks; t += gridDim.x * blockDim.x) {
   float p[6], C[21];
   int status = 0;

@@ -15,6 +15,7 @@
 // Global traffic per hit: one 8-byte read (plus an L2 re-read in the output pass) and a 12-byte
 // write (28 bytes with search records).
 #include "kf_math.cuh"
+#include "pdl.cuh"
 
 namespace kfgb {
 
@@ -27,6 +28,7 @@ __global__ void __launch_bounds__(1024, 2) k_build_hit_index(DevGeom G, const fl
                                                          int* __restrict__ sorted_ids, float4* __restrict__ sorted_rec,
                                                          uint4* __restrict__ sub_off, int* __restrict__ d_status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  pdl_begin();
   const int nb = G.n_bins;
   int* hist = reinterpret_cast<int*>(smem_raw);                       // [nb + 1]
   unsigned short* bin = reinterpret_cast<unsigned short*>(hist + nb + 1);  // [cap]
@@ -203,6 +205,7 @@ __global__ void __launch_bounds__(1024, 2)
                            float2* __restrict__ sorted_hits, int* __restrict__ sorted_ids, float4* __restrict__ sorted_rec,
                            uint4* __restrict__ sub_off, int* __restrict__ d_status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  pdl_begin();
   const int nb = G.n_bins;
   uint4* hist4 = reinterpret_cast<uint4*>(smem_raw);  // [nb]: the eight counters of each bin
   unsigned* hist = reinterpret_cast<unsigned*>(smem_raw);

@@ -7,6 +7,7 @@
 #include <algorithm>
 
 #include "mlp.cuh"
+#include "pdl.cuh"
 #include "tc.cuh"
 
 namespace kfgb {
@@ -250,6 +251,7 @@ __global__ void __launch_bounds__(fwd::kGroups* kGroup, 1) k_mlp_forward(const f
   const uint32_t h_off = fwd::H + gi * fwd::H_T;  // this group's X tile, then h1's lo part
   const int bid = gi + 1;
 
+  pdl_begin();
   stage_weights_b(params, S + fwd::W1, fwd::W1_T, S + fwd::W2, fwd::W2_T);
   if (threadIdx.x < kMlpHid) {
     b2[threadIdx.x] = params[kMlpB2 + threadIdx.x];
@@ -352,6 +354,7 @@ __global__ void __launch_bounds__(fwd::kGroups* kGroup, 1) k_mlp_forward(const f
 // m and K step s, lane l's four f16x2 words (rows 16 m + l / 4 and + 8, columns 16 s + 2 (l % 4)
 // and + 8; zero beyond the 14 inputs of the first layer), hi or scaled lo part.
 __global__ void k_mlp_fragments(const float* __restrict__ w, uint4* __restrict__ frag) {
+  pdl_begin();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < kFragWords; i += gridDim.x * blockDim.x) {
     const int part = i & 1, lane = (i >> 1) % 32;
     int m, s, ld;
@@ -384,7 +387,7 @@ __global__ void k_mlp_fragments(const float* __restrict__ w, uint4* __restrict__
 }
 
 int launch_mlp_fragments(const float* params, uint4* frag, cudaStream_t st) {
-  k_mlp_fragments<<<(kFragWords + 255) / 256, 256, 0, st>>>(params, frag);
+  launch_pdl(k_mlp_fragments, (kFragWords + 255) / 256, 256, 0, st, params, frag);
   return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
@@ -393,6 +396,7 @@ int launch_mlp_fragments(const float* params, uint4* frag, cudaStream_t st) {
 // candidate features and pulls; lanes 0-3 write the logits of rows 8w + 2l, 8w + 2l + 1.
 __global__ void k_mlp_finder_scores(const uint4* __restrict__ frag, const float* __restrict__ prm,
                                     const float* __restrict__ feats, int n, float* __restrict__ logits) {
+  pdl_begin();
   const int lane = threadIdx.x & 31;
   const long long r0 = (static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x) / 32 * 8;
   if (r0 >= n) return;  // whole warps leave together (r0 is the same for the warp's lanes)
@@ -417,7 +421,7 @@ int launch_mlp_finder_scores(const float* params, const float* feats, int n, flo
   if (launch_mlp_fragments(params, frag, st) != 0) return -3;
   if (n == 0) return 0;
   const long long warps = (static_cast<long long>(n) + 7) / 8;
-  k_mlp_finder_scores<<<static_cast<unsigned>((warps + 7) / 8), 256, 0, st>>>(frag, params, feats, n, logits);
+  launch_pdl(k_mlp_finder_scores, static_cast<int>((warps + 7) / 8), 256, 0, st, frag, params, feats, n, logits);
   return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
@@ -526,6 +530,7 @@ __global__ void __launch_bounds__(grd::kGroups* kGroup, 1)
   const uint32_t xh = grd::XH + gi * grd::XH_T;
   const int bid = gi + 1;
 
+  pdl_begin();
   stage_weights_b(params, S + grd::W1, grd::W1_T, S + grd::W2, grd::W2_T);
   if (threadIdx.x < kMlpHid) {
     b2[threadIdx.x] = params[kMlpB2 + threadIdx.x];
@@ -810,6 +815,7 @@ __global__ void __launch_bounds__(grd::kGroups* kGroup, 1)
 }
 
 __global__ void k_mlp_zero(float* grad, float* loss) {
+  pdl_begin();
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p < kMlpParams) grad[p] = 0.f;
   else if (p == kMlpParams) *loss = 0.f;
@@ -818,6 +824,7 @@ __global__ void k_mlp_zero(float* grad, float* loss) {
 // Adam (Kingma and Ba) on the weights; moments m, v; step t >= 1.
 __global__ void k_mlp_adam(float* params, const float* grad, float* m, float* v, int t, float lr, float b1, float b2,
                            float eps) {
+  pdl_begin();
   const float c1 = 1.f - powf(b1, static_cast<float>(t)), c2 = 1.f - powf(b2, static_cast<float>(t));
   for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < kMlpParams; p += gridDim.x * blockDim.x) {
     const float g = grad[p];
@@ -852,7 +859,7 @@ int launch_mlp_forward(const float* params, const float* feats, int n, float* lo
   int sms = 0;
   if (tc_prepare(reinterpret_cast<const void*>(k_mlp_forward), smem, &sms) != 0) return -3;
   const int tiles = (n + kTcM - 1) / kTcM;
-  k_mlp_forward<<<std::min(tiles, sms), fwd::kGroups * kGroup, smem, st>>>(params, feats, n, logits);
+  launch_pdl(k_mlp_forward, std::min(tiles, sms), fwd::kGroups * kGroup, smem, st, params, feats, n, logits);
   return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
@@ -861,16 +868,17 @@ int launch_mlp_loss_grad(const float* params, const float* feats, const float* l
   const int smem = static_cast<int>(grd::BYTES) + 1024;
   int sms = 0;
   if (tc_prepare(reinterpret_cast<const void*>(k_mlp_loss_grad), smem, &sms) != 0) return -3;
-  k_mlp_zero<<<(kMlpParams + 256) / 256, 256, 0, st>>>(grad, loss);
+  launch_pdl(k_mlp_zero, (kMlpParams + 256) / 256, 256, 0, st, grad, loss);
   const int tiles = (n + kTcM - 1) / kTcM;
   if (n > 0)
-    k_mlp_loss_grad<<<std::min(tiles, sms), grd::kGroups * kGroup, smem, st>>>(params, feats, labels, n, 1.f / n, grad, loss);
+    launch_pdl(k_mlp_loss_grad, std::min(tiles, sms), grd::kGroups * kGroup, smem, st, params, feats, labels, n, 1.f / n, grad,
+               loss);
   return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
 int launch_mlp_adam(float* params, const float* grad, float* m, float* v, int t, float lr, float b1, float b2, float eps,
                     cudaStream_t st) {
-  k_mlp_adam<<<(kMlpParams + 255) / 256, 256, 0, st>>>(params, grad, m, v, t, lr, b1, b2, eps);
+  launch_pdl(k_mlp_adam, (kMlpParams + 255) / 256, 256, 0, st, params, grad, m, v, t, lr, b1, b2, eps);
   return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
