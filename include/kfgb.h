@@ -230,9 +230,9 @@ int kf_fit_tracks(const KfGeometry* geom, const float* hits, const int* hit_surf
                   int* status_out, int block_threads, kf_stream_t stream);
 
 /* Device workspace (bytes) kf_find_tracks uses for these parameters on the current device. 4 bytes per
- * seed of it hold the order in which the seeds of a geometry with disks are taken (by direction,
- * which changes no result); a workspace without them is accepted and leaves the seeds in index
- * order. */
+ * seed of it hold the order in which the seeds are taken (by direction in a geometry with disks, else
+ * curling seeds first; it changes no result); a workspace without them is accepted and leaves the
+ * seeds in index order. */
 size_t kf_find_workspace_size(int n_seeds, const KfFindParams* params);
 
 /* Combinatorial track finding (Sec. 2 and Sec. 4): from each seed's three hits, fit the seed,

@@ -360,6 +360,7 @@ static int prepare_find(const KfGeometry* geom, const KfHitIndex* index, const f
   A->window_rank = params->mlp ? params->window_ranking : 0;
   A->seed_keep = params->seed_keep;
   A->class_count = nullptr;
+  A->front_list = nullptr;
   return KF_OK;
 }
 

@@ -431,6 +431,21 @@ __device__ __noinline__ bool load_seed_call(WarpSmem<KC>& W, int gbase, int slot
   return load_seed(W, gbase, slot, rec, surf_word);
 }
 
+// Seed number s of the order that takes the front list's seeds first and the others, which that list
+// has not marked (nor as removed or failed), in index order. Out of line: once per seed.
+static __device__ __noinline__ int front_seed(int s, int n, const int* front_list, const int* front_count,
+                                              const int* seed_surf, bool removed, int* counter) {
+  int nf = min(__ldg(front_count), n);
+  if (nf < n / 64) nf = 0;  // too few to wait for: as the others, in index order
+  if (s < nf) return front_list[s];
+  s -= nf;
+  if (nf > 0 || removed) {
+    const int mark = nf > 0 ? 3 : 2;  // bit 0: on the list, bit 1: removed or failed
+    while (s < n && ((seed_surf[s] >> 8) & mark) != 0) s = atomicAdd(counter, 1) - nf;
+  }
+  return s;
+}
+
 // Output of a finished seed: the best candidate (slot 0 of the group at gbase) and its hit list,
 // backtracked through the per-step trace of (parent slot, hit id + 1); the state and covariance
 // words are spread over the group's lanes. Out of line: once per seed.
@@ -536,6 +551,8 @@ __global__ void __launch_bounds__(LEARNED ? kFindMaxBlockLearned : 256, 2) k_fin
       s = atomicAdd(A.counter, 1);
       if (A.seed_list)  // second pass of adaptive capacity: the first pass's overflowing seeds
         s = s < min(*A.seed_list_count, n) ? A.seed_list[s] : n;
+      else if (A.front_list)
+        s = front_seed(s, n, A.front_list, A.front_count, A.seed_surf, A.seed_keep != nullptr, A.counter);
       else if (A.seed_keep)
         while (s < n && A.seed_keep[s] == 0) s = atomicAdd(A.counter, 1);
     }
@@ -563,7 +580,7 @@ __global__ void __launch_bounds__(LEARNED ? kFindMaxBlockLearned : 256, 2) k_fin
     // ---- a fresh group loads its seed state into slot 0 ------------------------------------
     if (fresh) {
       // Candidate surface word: (position in the region's list + 1) << 8 | surface.
-      const int s3 = A.seed_surf[seed];
+      const int s3 = A.seed_surf[seed] & 255;
       int pos = -1;
       if (STEER && G.steer && s3 >= 0 && s3 < G.n_surf) {
         region = seed_region(G, s3, A.hits[A.seed_hits[static_cast<size_t>(2) * n + seed]]);

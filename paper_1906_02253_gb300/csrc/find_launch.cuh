@@ -39,6 +39,8 @@ struct FindArgs {
   float* seed_state;  // [28][n_seeds]: p[6], C[21], chi2 (< 0: failed seed)
   int* seed_surf;     // [n_seeds]: surface of the third seed hit
   int* class_count;   // seeds of each direction class (the seed-state kernel counts them), or null
+  int* front_list;    // seeds taken before the others (the seed-state kernel lists them), or null
+  int* front_count;
   // Adaptive capacity (plain finding): a first pass at a smaller capacity (detect = 1) finishes the
   // seeds whose children never outnumber its slots, which then have exactly the results of the
   // full capacity, and lists the others in ovf_list (*ovf_count of them) without writing their

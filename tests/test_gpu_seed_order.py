@@ -1,6 +1,6 @@
-"""Finding with the seeds taken by direction (geometries with disks, a workspace of the full size) gives
-bit for bit what it gives with the seeds in index order (a workspace without the order's 4 bytes per
-seed), at the edges of the ordering kernel's blocks, with failed and removed seeds, in one pass and
+"""Finding with the seeds taken in the library's own order (by direction in geometries with disks, curling
+seeds first in the others; a workspace of the full size) gives bit for bit what it gives with the
+seeds in index order (a workspace without the order's 4 bytes per seed), at the edges of the ordering kernel's blocks, with failed and removed seeds, in one pass and
 two, plain, learned and with options."""
 import ctypes
 import os
@@ -30,18 +30,29 @@ def batch(kf):
     return wl, kf.to_device_event_batch(b)
 
 
+@pytest.fixture(scope="module")
+def barrel(kf):
+    """Barrel seeds, the odd ones of hits of different particles, which curl."""
+    wl = synth.workload("find", n_events=2, tracks_lo=2300, tracks_hi=2300, seed=18)
+    dev = kf.to_device_event_batch(synth.generate(wl))
+    dev["seed_hits"][1, 1::2] = dev["seed_hits"][1, 1::2].roll(1)
+    return wl, dev
+
+
 def _up(v):
     return (v + 255) // 256 * 256
 
 
 @pytest.mark.parametrize("n", [1, 2, 127, 128, 129, 2047, 2048, 2049, 4600])
-@pytest.mark.parametrize("option", ["plain", "two_passes", "learned", "field"])
-def test_order_changes_no_result(kf, batch, n, option):
-    wl, dev = batch
+@pytest.mark.parametrize("option", ["plain", "two_passes", "learned", "field", "barrel", "barrel_all_kept", "barrel_few_curl"])
+def test_order_changes_no_result(kf, batch, barrel, n, option):
+    wl, dev = barrel if option.startswith("barrel") else batch
     from dataclasses import replace
     g = kf.Geometry(wl if option == "field" else replace(wl, field_z2=0.0, field_r2=0.0))
     ix = kf.build_hit_index(g, dev["hits"], dev["slab_offsets"], 2, dev["max_slab_hits"])
     some = torch.linspace(0, dev["seed_hits"].shape[1] - 1, n).long().cuda()
+    if option == "barrel_few_curl":  # below the share from which they go first
+        some[10:] = some[10:] // 2 * 2
     seeds, event = dev["seed_hits"][:, some].contiguous(), dev["seed_event"][some].contiguous()
     keep = torch.ones(n, dtype=torch.int32, device="cuda")
     if n > 10:
@@ -49,6 +60,8 @@ def test_order_changes_no_result(kf, batch, n, option):
         seeds[:, 5] = seeds[0, 5]  # failed: one hit three times
         event[7] = 9              # failed: no such event
         keep[::6] = 0             # removed by cleaning
+    if option == "barrel_all_kept":
+        keep = None
     net = None
     if option == "learned":
         z = np.load(os.path.join(os.path.dirname(kf.__file__), "data", "mlp_hi_occ.npz"))
@@ -74,11 +87,15 @@ def test_order_changes_no_result(kf, batch, n, option):
     a, b = outs
     for k in a:
         assert torch.equal(a[k].view(torch.int32), b[k].view(torch.int32)), k
+    keep = torch.ones(n, dtype=torch.int32, device="cuda") if keep is None else keep
     want = torch.where(keep == 0, 2, 0)
     if n > 10:
         for i in (3, 5, 7):
             want[i] = 1 if keep[i] else 2
-    assert torch.equal(a["status"], want.to(torch.int32))
+    if option.startswith("barrel"):  # seeds of hits of different particles may fail as well
+        assert torch.equal(a["status"] == 2, keep == 0)
+    else:
+        assert torch.equal(a["status"], want.to(torch.int32))
     # a smaller one is refused
     rc = kf.load_library().kf_find_tracks(
         g.ref, ctypes.byref(ix.c), P(dev["hits"]), P(dev["hit_surface"]), P(seeds), P(event), n, ctypes.byref(prm), P(out["hits"]),
