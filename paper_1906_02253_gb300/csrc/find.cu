@@ -109,7 +109,8 @@ __global__ void __launch_bounds__(128) k_seed_states(DevGeom G, const __grid_con
     mark = (front ? 1 : 0) | (live ? 0 : 2);  // passed over in index order
   }
   if (!in) return;
-  if (ok || A.class_count || A.front_list) A.seed_surf[seed] = ss[2] | (mark << 8);
+  // (a failed seed has no surface: 255, above every surface's number, so that nothing looks its hits up)
+  if (FIND || ok) A.seed_surf[seed] = (ok ? ss[2] : 255) | (mark << 8);
   if constexpr (FIND) {
     float* out = A.seed_state + static_cast<size_t>(seed) * kSeedWords;
     if (ok) {
@@ -415,6 +416,7 @@ int launch_find(const DevGeom& G, const DevMat& M, FindArgs& A, const FindPlan& 
   // [3] the number of seeds in the ordered list, [4] in the front list, [8 ...] the classes' counts, [32 ...]
   // their cursors. (A kernel clears them because a memset would not start under the kernel before.)
   constexpr int kCounters = 56;
+  static_assert(kMaxSurf <= 255, "surface numbers share a word with a mark");
   static_assert(8 + kClasses <= 32 && 32 + kClasses <= kCounters && kCounters * sizeof(int) <= 256, "counter area");
   const bool disks = G.n_dpos + G.n_dneg > 0, room = ws_bytes >= plan.ws_bytes, ordered = disks && room;
   int* list = reinterpret_cast<int*>(base + plan.off_order);

@@ -44,7 +44,8 @@ def _up(v):
 
 
 @pytest.mark.parametrize("n", [1, 2, 127, 128, 129, 2047, 2048, 2049, 4600])
-@pytest.mark.parametrize("option", ["plain", "two_passes", "learned", "field", "barrel", "barrel_all_kept", "barrel_few_curl"])
+@pytest.mark.parametrize("option", ["plain", "two_passes", "learned", "field", "barrel", "barrel_all_kept", "barrel_few_curl",
+                                    "barrel_steered"])
 def test_order_changes_no_result(kf, batch, barrel, n, option):
     wl, dev = barrel if option.startswith("barrel") else batch
     from dataclasses import replace
@@ -66,7 +67,13 @@ def test_order_changes_no_result(kf, batch, barrel, n, option):
     if option == "learned":
         z = np.load(os.path.join(os.path.dirname(kf.__file__), "data", "mlp_hi_occ.npz"))
         net = kf.mlp_buffer(z["weights"], z["mean"], z["sd"])
-    prm = kf.find_params(wl.chi2_cut, wl.k_max, wl.max_miss, wl.lmax, seed_keep=keep, mlp=net, top_n=2 if net is not None else 0,
+    layers = list(range(len(wl.surfaces)))
+    steer = dict(c_barrel=0.4, c_endcap=3.0, lists=[layers] * 5) if option == "barrel_steered" else None
+    if steer:  # failed seeds without removed ones, and a failed seed whose third hit is the missing one
+        keep = None
+        if n > 10:
+            seeds[2, 9] = -1
+    prm = kf.find_params(wl.chi2_cut, wl.k_max, wl.max_miss, wl.lmax, seed_keep=keep, steering_tables=steer, mlp=net, top_n=2 if net is not None else 0,
                          score_margin=0.7 if net is not None else 0.0, adaptive_capacity=2 if option == "two_passes" else 0)
     full = kf.find_workspace_size(n, prm)
     room = torch.empty(full, dtype=torch.uint8, device="cuda")
