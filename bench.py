@@ -72,15 +72,15 @@ FIND_SOURCES = ("paper_1906_02253_gb300/csrc/find.cu", "paper_1906_02253_gb300/c
                 "paper_1906_02253_gb300/csrc/find_learned.cu", "paper_1906_02253_gb300/csrc/kf_math.cuh",
                 "paper_1906_02253_gb300/csrc/find_launch.cuh", "paper_1906_02253_gb300/csrc/mlp.cuh",
                 "paper_1906_02253_gb300/build.py")
-FIND_PROFILE = {"sources_sha1": "37e3a4f5b5505e80f57304bd1472dadac3fc4110",
-                "dram_bytes_per_seed": {"fit_100ev_uneven_17layers_ms": (125605888 + 35233024) / 302063,
-                                        "find_200ev_barrel_disks_noise100": (144240128 + 31036672) / 211523,
+FIND_PROFILE = {"sources_sha1": "e7656bf397b4a70bd709c2e54333c0d224d91176",
+                "dram_bytes_per_seed": {"fit_100ev_uneven_17layers_ms": (124858112 + 34387968) / 302063,
+                                        "find_200ev_barrel_disks_noise100": (231109376 + 69856768) / 211523,
                                         "find_200ev_barrel_disks_noise100_adaptive4":
-                                            (170531328 + 35969024 + 128829952 + 27841280) / 211523,
+                                            (223592192 + 64325632 + 124954368 + 34751232) / 211523,
                                         "find_200ev_barrel_disks_noise100_adaptive2":
-                                            (168316416 + 38796544 + 159785216 + 35333632) / 211523,
+                                            (206157568 + 55670272 + 181676800 + 49921280) / 211523,
                                         "find_200ev_barrel_disks_noise100_adaptive2_learned2_0.7":
-                                            (154265088 + 31579648 + 42024960 + 3967232) / 211523}}
+                                            (236084480 + 68200448 + 29479936 + 3928576) / 211523}}
 # Hit index: algorithmic HBM bytes per hit (read 8 B of (phi, z); write 8 B sorted, 4 B id, 16 B search
 # record) plus, per (event, surface), the bin offsets (4 B per bin + 1) and the phi sub-bin offsets (16 B per bin).
 INDEX_BYTES_PER_HIT = 36
@@ -393,11 +393,13 @@ def measure_workload(args, wl, batch, full: bool = True, mlp_name: str = None, e
         dist.barrier()
     from paper_1906_02253_gb300 import shard
     ms_step = shard.max_over_ranks(statistics.mean(t_steps), device=dev)
-    # index, seed states, find, fit kernels (plus one memset node); adaptive capacity: a second find
-    # pass; cleaning: count, 3 scan kernels, fill, seed directions, decision; duplicate removal:
-    # count, 3 scan kernels, fill, decision
+    # index, counters' clearing, seed states, find, fit kernels; with disks the seeds' ordering by
+    # direction; adaptive capacity: a second find pass; cleaning: count, 3 scan kernels, fill, seed
+    # directions, decision; duplicate removal: count, 3 scan kernels, fill, decision;
     # learned proposal: the weight-fragment kernel before the finder
-    launches_per_step = 4 + (1 if prm.adaptive_capacity > 0 else 0) + (7 + 6 if clean else 0) + (1 if lrn else 0)
+    ordered = any(s.type == synth.DISK for s in batch.wl.surfaces)
+    launches_per_step = (5 + (1 if ordered else 0) + (1 if prm.adaptive_capacity > 0 else 0) + (7 + 6 if clean else 0)
+                         + (1 if lrn else 0))
 
     # Per-part durations: the same launches eager, events on the launching stream.
     kern = {k: [] for k in parts}

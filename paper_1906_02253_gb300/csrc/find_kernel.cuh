@@ -14,14 +14,16 @@
 //     below the cut are buffered in flattened order, so each owner's pairs form one contiguous
 //     run, which the owner merges into its list of the k_max best by (total chi2, hit id);
 //  3. per seed, each lane offers its children (hit children, miss child, carried candidate) as a
-//     sorted list; k_max rounds of a tournament over the lists' heads (a segmented minimum by
-//     shuffles) rank them, the child of rank j goes to slot j, and lane j materialises it (Kalman
-//     update for a hit child) from its parent's record;
+//     sorted list; they are ranked by counting (plain instances without options: every child
+//     compares its key with the group's) or by k_max rounds of a tournament over the lists' heads
+//     (the others: a segmented minimum by shuffles). The child of rank j goes to slot j, and lane j
+//     materialises it (Kalman update for a hit child) from its parent's record;
 //  4. a seed whose candidates have all stopped writes its best track (backtracking a per-step
 //     trace of parent slot and hit) and its lanes take the next seed from an atomic queue.
 // The warps of a block vote once per step (block barrier), which keeps them in the same phase.
-// Seeds are consumed in queue order, one event after another, so the warps of the GPU read the
-// index of one or two events at a time through L2.
+// Without disks seeds are consumed in index order, one event after another, so the warps of the GPU
+// read the index of one or two events at a time through L2 (strongly curled seeds first where there
+// are many); with disks by direction class, so that a block's seeds cross alike surfaces (find.cu).
 #pragma once
 
 #include <algorithm>

@@ -189,7 +189,7 @@ __global__ void __launch_bounds__(1024, 2) k_build_hit_index(DevGeom G, const fl
 // histogram counts fine bins (two 16-bit counters a word), so its scan yields the sub-bin offsets
 // and the bin offsets at once, a hit's rank is searched only among the hits of its own fine bin
 // (0.2 to 1.2 on average here, 2 to 10 in its bin), and a hit keeps one 16-bit word instead of a
-// bin and a sub-bin. 200 barrel + disk events (28.6 M hits, 7,000 slabs) take 437 us against 466 us
+// bin and a sub-bin. 200 barrel + disk events (28.6 M hits, 7,000 slabs) take 434 us against 466 us
 // with bins and sub-bins apart, the search records 55 us of it; issue and latency bound (a slab is a
 // chain of eight block barriers). 512 or 768 threads a block are 2-3% slower, as the largest slab's
 // shared memory keeps it at two blocks per SM.

@@ -60,7 +60,7 @@ __device__ __forceinline__ void parts_to_smem(unsigned char* t0, int row, int ha
 // relu(D1) -> the next A operand (in D1's columns; its lo part over the X tile, which the finished
 // MMA no longer needs); D2 = H W2^T; logit = b3 + sum_j W3[j] relu(D2[j] + b2[j]) on the CUDA cores.
 // Four groups per CTA (1024 threads at 64 registers, all 512 tensor-memory columns). 1,000,003 rows take
-// 55 us (183 TFLOP/s of the network's flops, six times that on the tensor cores: 58% of the measured
+// 53 us (192 TFLOP/s of the network's flops, six times that on the tensor cores: 60% of the measured
 // bf16 rate), where one chain per CTA, two CTAs per SM, took 115 us; the bound is the CUDA cores'
 // issue rate (splits, ReLU, output layer), then the tensor pipe.
 namespace fwd {
@@ -445,9 +445,9 @@ int launch_mlp_finder_scores(const float* params, const float* feats, int n, flo
 // gradient MMAs; the other group then runs its layers.
 // Tensor memory: per group D1, then h1, then e2 (parts_to_tmem) at 0, D2 then D3 at 96; Dg2 at 320,
 // Dg1 at 464.
-// 2,000,003 rows take 415 us (137 TFLOP/s of the network's flops), where one group per CTA took 895 us;
+// 2,000,003 rows take 408 us (139 TFLOP/s of the network's flops), where one group per CTA took 895 us;
 // the bound is the tensor pipe fetching operands (a gradient MMA with an MN-major A of 128 rows takes 70
-// to 96 cycles). A step's 4,096 rows: kernels 21 us against 85 us; their tile, prologue and epilogue
+// to 96 cycles). A step's 4,096 rows: the whole step 18 us against 98 us; their tile, prologue and epilogue
 // are one chain (the old epilogue added 32 lanes to one shared-memory float, a CAS loop each).
 namespace grd {
 constexpr int kGroups = 2;
