@@ -199,12 +199,14 @@ __device__ __forceinline__ auto mnmajor(uint32_t base) {
   return Operand<KT / 8 * 128u, 128u, 2u * (KT / 8 * 128u)>(base);
 }
 
-// D = A B^T over one K = 16 step as the six products of the three-part split (hi*hi, hi*mid,
-// mid*hi, hi*lo, lo*hi, mid*mid); the parts of A and B lie AT and BT bytes apart. One thread issues,
-// the mbarrier receives the completion.
+// D = A B^T over one K = 16 step as the six products of the three-part split, the smallest first
+// (lo*hi, hi*lo, mid*mid, mid*hi, hi*mid, hi*hi); the parts of A and B lie AT and BT bytes apart. One
+// thread issues, the mbarrier receives the completion. The order costs nothing (the same MMAs) and the
+// tensor pipe's rounding of the FP32 accumulator then falls on small sums: with hi*hi first the logits'
+// error against FP64 was 7.4e-7 of the largest, with it last, here and over K = 64, it is 1.7e-7.
 template <uint32_t AT, uint32_t BT, class OA, class OB>
 __device__ __forceinline__ void mma_split16(uint32_t d, const OA& A, const OB& B, uint32_t idesc, uint64_t* bar) {
-  constexpr int kPa[6] = {0, 0, 1, 0, 2, 1}, kPb[6] = {0, 1, 0, 2, 0, 1};
+  constexpr int kPa[6] = {2, 0, 1, 1, 0, 0}, kPb[6] = {0, 2, 1, 0, 1, 0};
   tc::fence_after_sync();
 #pragma unroll
   for (int p = 0; p < 6; ++p) tc::mma_bf16(d, A.at(AT * kPa[p], 0), B.at(BT * kPb[p], 0), idesc, p > 0 ? 1u : 0u);
@@ -212,7 +214,8 @@ __device__ __forceinline__ void mma_split16(uint32_t d, const OA& A, const OB& B
 }
 
 // D = A B^T over K = 64 with A's parts in tensor memory (columns from region as parts_to_tmem lays
-// them), or (LO = false) its lo part, which one of the six products reads, in shared memory.
+// them), or (LO = false) its lo part, which one of the six products reads, in shared memory. The hi*hi
+// products of all four K steps come last.
 template <bool LO, uint32_t BT, class OL, class OB>
 __device__ __forceinline__ void mma_split_ta(uint32_t d, uint32_t region, const OL& lo, const OB& B, uint32_t idesc,
                                              uint64_t* bar) {
@@ -220,14 +223,15 @@ __device__ __forceinline__ void mma_split_ta(uint32_t d, uint32_t region, const 
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     const uint32_t ah = region + 32 * (k >> 1) + 8 * (k & 1), am = ah + 16;
-    tc::mma_bf16_ta(d, ah, B.at(0, k), idesc, k > 0 ? 1u : 0u);
-    tc::mma_bf16_ta(d, ah, B.at(BT, k), idesc, 1u);
-    tc::mma_bf16_ta(d, am, B.at(0, k), idesc, 1u);
+    if constexpr (LO) tc::mma_bf16_ta(d, region + 64 + 8 * k, B.at(0, k), idesc, k > 0 ? 1u : 0u);
+    else tc::mma_bf16(d, lo.at(0, k), B.at(0, k), idesc, k > 0 ? 1u : 0u);
     tc::mma_bf16_ta(d, ah, B.at(2 * BT, k), idesc, 1u);
-    if constexpr (LO) tc::mma_bf16_ta(d, region + 64 + 8 * k, B.at(0, k), idesc, 1u);
-    else tc::mma_bf16(d, lo.at(0, k), B.at(0, k), idesc, 1u);
     tc::mma_bf16_ta(d, am, B.at(BT, k), idesc, 1u);
+    tc::mma_bf16_ta(d, am, B.at(0, k), idesc, 1u);
+    tc::mma_bf16_ta(d, ah, B.at(BT, k), idesc, 1u);
   }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) tc::mma_bf16_ta(d, region + 32 * (k >> 1) + 8 * (k & 1), B.at(0, k), idesc, 1u);
   tc::mma_commit(bar);
 }
 
