@@ -975,7 +975,9 @@ __global__ void __launch_bounds__(LEARNED ? kFindMaxBlockLearned : 256, 2) k_fin
       const int all = __shfl_sync(kFull, cincl, in_grp ? gbase + KC - 1 : lane), tot = in_grp ? all : 0;
       ovf = detect && tot > KC;
       const int first = cincl - nch;  // number of this lane's first child
-      if (ovf) nch = 0;
+      // A detecting pass with more slots than k_max counts passing hits that no list keeps: they make the
+      // seed overflow, but are not offered (their numbers stay empty below).
+      nch = ovf ? 0 : kind == 0 ? min(nch, hl_n) : nch;
       const int most = static_cast<int>(__reduce_max_sync(kFull, ovf ? 0 : tot));
       unsigned long long* const kb = W.u.key + (in_grp ? grp * 2 * KC : 0);
       auto gather = [&](int c0, int c1, int at) {  // children numbered [c0, c1) to kb[at ...]
