@@ -247,9 +247,9 @@ size_t kf_find_workspace_size(int n_seeds, const KfFindParams* params);
  * hit marking across seeds (Sec. 3.2).
  *   hits, hit_surface  as for the fit (original hit ids); index built by kf_build_hit_index.
  *   seed_hits          device int [3][n_seeds] (structure of arrays), seed_event int [n_seeds]. A
- *                      seed with a negative hit id, a hit on no surface of the geometry or an event
- *                      outside [0, index->n_events) fails (status 1); hit ids must be below the
- *                      number of hits.
+ *                      seed with a negative hit id, a hit on no surface of the geometry, an event
+ *                      outside [0, index->n_events) or a fit whose chi2 is below zero or NaN fails
+ *                      (status 1); hit ids must be below the number of hits.
  *   workspace          device memory of kf_find_workspace_size bytes, 256-byte aligned, owned
  *                      by this call until its kernels finish: calls that can run at the same time
  *                      (other streams, other host threads) need workspaces of their own (sharing
@@ -270,7 +270,7 @@ int kf_find_tracks(const KfGeometry* geom, const KfHitIndex* index, const float*
  *                          another event fails).
  *   state_out  device float [28][n_seeds] (structure of arrays): p[6], packed C[21] at hit 3 and
  *              chi2 (sum of the three predicted chi2); chi2 = -1 marks a seed that failed (invalid
- *              hit id, event or surface, collinear hits, no crossing).
+ *              hit id, event or surface, collinear hits, no crossing, a chi2 below zero or NaN).
  *   surf_out   device int [n_seeds]: surface of hit 3 (set for seeds that did not fail).
  * Asynchronous on the stream; KF_ERR_ARG for a bad geometry, negative counts or null pointers. */
 int kf_seed_states(const KfGeometry* geom, const float* hits, const int* hit_surface, const int* seed_hits,

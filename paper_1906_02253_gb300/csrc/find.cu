@@ -80,6 +80,9 @@ __global__ void __launch_bounds__(128) k_seed_states(DevGeom G, const __grid_con
     const float2 h = A.hits[ids[k]];
     c.chi2 += update_exact(G, ss[k], c, h.x, h.y);
   }
+  // One predicate for "the finder takes it" and "its outputs are written here": a chi2 that is NaN (a hit
+  // with a NaN coordinate) or negative (a covariance that lost its sign in FP32) marks no state.
+  ok = ok && c.chi2 >= 0.f;
   // With an order to make: the class of a seed the finder will take (k_order_seeds reads it from
   // above the surface), counted per block and added once.
   int cls = -1;
@@ -87,7 +90,7 @@ __global__ void __launch_bounds__(128) k_seed_states(DevGeom G, const __grid_con
     __shared__ int hist[kClasses];
     if (threadIdx.x < kClasses) hist[threadIdx.x] = 0;
     __syncthreads();
-    if (ok && c.chi2 >= 0.f) {
+    if (ok) {
       cls = seed_class(c.p[5]);
       atomicAdd(&hist[cls], 1);
     }
@@ -96,8 +99,7 @@ __global__ void __launch_bounds__(128) k_seed_states(DevGeom G, const __grid_con
   }
   int mark = A.class_count ? cls + 1 : 0;
   if (A.front_list) {
-    const bool live = ok && c.chi2 >= 0.f;
-    const bool front = live && fabsf(kCurvF * G.bz * c.p[3]) * G.barrel_r[G.n_barrel - 1] > kCurling;
+    const bool front = ok && fabsf(kCurvF * G.bz * c.p[3]) * G.barrel_r[G.n_barrel - 1] > kCurling;
     const unsigned mask = __ballot_sync(kFull, front);
     if (mask) {
       const int lane = threadIdx.x & 31;
@@ -106,7 +108,7 @@ __global__ void __launch_bounds__(128) k_seed_states(DevGeom G, const __grid_con
       at = __shfl_sync(kFull, at, __ffs(mask) - 1) + __popc(mask & ((1u << lane) - 1u));
       if (front && at < n) A.front_list[at] = seed;
     }
-    mark = (front ? 1 : 0) | (live ? 0 : 2);  // passed over in index order
+    mark = (front ? 1 : 0) | (ok ? 0 : 2);  // passed over in index order
   }
   if (!in) return;
   // (a failed seed has no surface: 255, above every surface's number, so that nothing looks its hits up)

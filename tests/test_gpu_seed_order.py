@@ -43,6 +43,51 @@ def _up(v):
     return (v + 255) // 256 * 256
 
 
+def _all_written(out, n_hits):
+    """Every seed has outputs: nothing of the -7 that the buffers held, no hit id outside the hits."""
+    assert ((out["status"] >= 0) & (out["status"] <= 2)).all()
+    assert (out["nhits"] >= 0).all()
+    assert ((out["hits"] >= -1) & (out["hits"] < n_hits)).all()
+    bad = out["status"] != 0
+    assert (out["hits"][:, bad] == -1).all() and (out["nhits"][bad] == 0).all()
+    assert out["chi2"][bad].isnan().all() and out["state"][:, bad].isnan().all() and out["cov"][:, bad].isnan().all()
+
+
+@pytest.mark.parametrize("option", ["disks", "barrel", "barrel_static"])
+def test_a_seed_whose_fit_gives_no_chi2_fails(kf, batch, barrel, option):
+    """A NaN coordinate of a seed's second or third barrel hit leaves its circle as it is and makes the
+    chi2 NaN: the seed fails, and its outputs say so."""
+    wl, dev = batch if option == "disks" else barrel
+    g = kf.Geometry(wl)
+    hits = dev["hits"].clone()
+    ids = dev["seed_hits"].long()
+    on_barrel = (dev["hit_surface"][ids[1]] < 17) & (dev["hit_surface"][ids[2]] < 17)
+    some = torch.nonzero(on_barrel).squeeze(1)[5:2000:20]
+    hits[ids[1, some[0::2]], 1] = float("nan")
+    hits[ids[2, some[1::2]], 1] = float("nan")
+    ix = kf.build_hit_index(g, hits, dev["slab_offsets"], 2, dev["max_slab_hits"])
+    n = ids.shape[1]
+    out = dict(hits=torch.full((wl.lmax, n), -7, dtype=torch.int32, device="cuda"))
+    for k in ("nhits", "status"):
+        out[k] = torch.full((n,), -7, dtype=torch.int32, device="cuda")
+    out["chi2"] = torch.full((n,), -7.0, device="cuda")
+    out["state"], out["cov"] = torch.full((6, n), -7.0, device="cuda"), torch.full((21, n), -7.0, device="cuda")
+    prm = kf.find_params(wl.chi2_cut, wl.k_max, wl.max_miss, wl.lmax)
+    if option == "barrel_static":
+        P = lambda t: ctypes.c_void_p(t.data_ptr())  # noqa: E731
+        rc = kf.load_library().kf_find_tracks_static(
+            g.ref, ctypes.byref(ix.c), P(hits), P(dev["hit_surface"]), P(dev["seed_hits"]), P(dev["seed_event"]), n,
+            ctypes.byref(prm), P(out["hits"]), P(out["nhits"]), P(out["chi2"]), P(out["state"]), P(out["cov"]), P(out["status"]),
+            ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+        assert rc == kf.KF_OK
+    else:
+        kf.find_tracks(g, ix, hits, dev["hit_surface"], dev["seed_hits"], dev["seed_event"], prm, out=out)
+    _all_written(out, hits.shape[0])
+    assert len(some) > 50 and (out["status"][some] == 1).all()
+    state, _ = kf.seed_states(g, hits, dev["hit_surface"], dev["seed_hits"], dev["seed_event"], 2)
+    assert torch.equal(state[27] < 0, out["status"] != 0) and not state[27].isnan().any()
+
+
 @pytest.mark.parametrize("n", [1, 2, 127, 128, 129, 2047, 2048, 2049, 4600])
 @pytest.mark.parametrize("option", ["plain", "two_passes", "learned", "field", "barrel", "barrel_all_kept", "barrel_few_curl",
                                     "barrel_steered"])
@@ -94,6 +139,7 @@ def test_order_changes_no_result(kf, batch, barrel, n, option):
     a, b = outs
     for k in a:
         assert torch.equal(a[k].view(torch.int32), b[k].view(torch.int32)), k
+    _all_written(a, dev["hits"].shape[0])
     keep = torch.ones(n, dtype=torch.int32, device="cuda") if keep is None else keep
     want = torch.where(keep == 0, 2, 0)
     if n > 10:
