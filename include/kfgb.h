@@ -345,7 +345,8 @@ int kf_mlp_finder_scores(const float* params, const float* features, int n, floa
  * respect to the KF_MLP_PARAMS weights: grad float [KF_MLP_PARAMS] and loss float [1] are
  * overwritten. Features as for kf_mlp_forward (8-byte aligned). The forward layers, the
  * back-propagation through W2 and the weight gradients of W1, b1, W2, b2 run on the tensor cores
- * with the same FP32-faithful split; a tensor-core wait that gives up makes the loss NaN. */
+ * with the same FP32-faithful split; a tensor-core wait that gives up makes the loss NaN, and its block
+ * adds nothing to the gradient. */
 int kf_mlp_loss_grad(const float* params, const float* features, const float* labels, int n, float* grad,
                      float* loss, kf_stream_t stream);
 
@@ -429,6 +430,12 @@ int kf_math_probe(int fn, const float* a, const float* b, int n, float* o0, floa
  * wait's duration in ns); expected (0, 1, about limit_us * 1000). KF_ERR_ARG for limit_us outside
  * [1, 1000000] or a null pointer. */
 int kf_wait_probe(int limit_us, long long* out, kf_stream_t stream);
+
+/* Probe of what a wait that gives up leaves in kf_mlp_loss_grad's outputs (measurement only): the same
+ * call, but the block that takes tile `tile` (rows 128 tile .. 128 tile + 127) treats its wait for the
+ * second layer there as given up. KF_ERR_ARG as kf_mlp_loss_grad, and for a tile < 0. */
+int kf_mlp_wait_probe(const float* params, const float* features, const float* labels, int n, int tile, float* grad,
+                      float* loss, kf_stream_t stream);
 
 /* Human-readable name of a status code. */
 const char* kf_status_string(int status);

@@ -68,7 +68,7 @@ EXPORTS = ("kf_build_hit_index", "kf_index_bins", "kf_fit_tracks", "kf_find_work
            "kf_find_tracks_static", "kf_mlp_forward", "kf_mlp_loss_grad", "kf_mlp_adam", "kf_autotune_find",
            "kf_autotune_fit", "kf_status_string", "kf_dedup_workspace_size", "kf_clean_seeds",
            "kf_remove_duplicates", "kf_fp32_fma_probe", "kf_math_probe", "kf_seed_states",
-           "kf_wait_probe", "kf_mlp_finder_scores")
+           "kf_wait_probe", "kf_mlp_finder_scores", "kf_mlp_wait_probe")
 MLP_PARAMS, MLP_BUFFER = 5185, 5213
 KF_MLP_FRAG_BYTES = 20480  # the finder's tensor-core operands of the network (kfgb.h)
 PHI_SUB = 8  # KF_PHI_SUB: phi sub-bins per phi bin of the hit index
@@ -125,6 +125,8 @@ def load_library(path: str = LIB_PATH):
             lib.kf_math_probe.argtypes = [I, P, P, I, P, P, P, P]
             lib.kf_wait_probe.restype = I
             lib.kf_wait_probe.argtypes = [I, P, P]
+            lib.kf_mlp_wait_probe.restype = I
+            lib.kf_mlp_wait_probe.argtypes = [P, P, P, I, I, P, P, P]
             lib.kf_status_string.restype = ctypes.c_char_p
             lib.kf_status_string.argtypes = [I]
             _lib = lib
@@ -362,6 +364,16 @@ def wait_probe(limit_us: int, stream=None):
     out = torch.full((3,), -1, dtype=torch.int64, device="cuda")
     _check(load_library().kf_wait_probe(int(limit_us), _ptr(out), _stream(stream)), "kf_wait_probe")
     return out
+
+
+def mlp_wait_probe(params, features, labels, tile: int, stream=None):
+    """kf_mlp_wait_probe: mlp_loss_grad with the tensor-core wait of one tile treated as given up."""
+    for t, name in ((params, "params"), (features, "features"), (labels, "labels")):
+        _cuda(t, torch.float32, name)
+    grad, loss = torch.empty(MLP_PARAMS, device=params.device), torch.empty(1, device=params.device)
+    _check(load_library().kf_mlp_wait_probe(_ptr(params), _ptr(features), _ptr(labels), features.shape[0], int(tile),
+                                            _ptr(grad), _ptr(loss), _stream(stream)), "kf_mlp_wait_probe")
+    return loss, grad
 
 
 def math_probe(fn: int, a, b=None, stream=None):

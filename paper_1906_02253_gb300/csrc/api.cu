@@ -433,6 +433,13 @@ int kf_mlp_loss_grad(const float* params, const float* features, const float* la
   return launch_mlp_loss_grad(params, features, labels, n, grad, loss, reinterpret_cast<cudaStream_t>(stream));
 }
 
+int kf_mlp_wait_probe(const float* params, const float* features, const float* labels, int n, int tile, float* grad,
+                      float* loss, kf_stream_t stream) {
+  if (n < 0 || tile < 0 || !params || !grad || !loss || (n > 0 && (!features || !labels))) return KF_ERR_ARG;
+  if (reinterpret_cast<size_t>(features) & 7) return KF_ERR_ARG;
+  return launch_mlp_wait_probe(params, features, labels, n, grad, loss, tile, reinterpret_cast<cudaStream_t>(stream));
+}
+
 int kf_mlp_adam(float* params, const float* grad, float* m, float* v, int step, float lr, float beta1, float beta2,
                 float eps, kf_stream_t stream) {
   if (!params || !grad || !m || !v || step < 1 || !(lr > 0.f) || !(eps > 0.f)) return KF_ERR_ARG;

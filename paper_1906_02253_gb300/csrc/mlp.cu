@@ -460,7 +460,7 @@ constexpr int kHm = 0, kHh = 8, kXh = 16, kXm = 18, kXl = 20, kHl = 22;  // 8-co
 constexpr uint32_t E_T = kTcM * kEK * 2, XH_T = kTcM * kXhK * 2, W1_T = 2048, W2_T = 8192;  // bytes of one tile
 constexpr uint32_t E = 0, XH = E + E_T, W2 = XH + kGroups * XH_T, W1 = W2 + 3 * W2_T, B2 = W1 + 3 * W1_T,
                    W3 = B2 + 256, MEAN = W3 + 256, SD = MEAN + 64, RS = SD + 64, PART = RS + 64, RED = PART + kGroups * 1024,
-                   BAR = RED + 16 * 34 * 4, TMEM = BAR + 16 * kGroups, LOCK = TMEM + 4, USED = LOCK + 4, BYTES = USED + 8;
+                   BAR = RED + 16 * 34 * 4, TMEM = BAR + 16 * kGroups, LOCK = TMEM + 4, USED = LOCK + 4, FAILED = USED + 4, BYTES = FAILED + 8;
 static_assert(BYTES + 1024 <= 227 * 1024, "shared-memory layout");
 constexpr uint32_t kCols = 512, kColD2 = 96, kColG2 = 320, kColG1 = 464;
 }  // namespace grd
@@ -509,9 +509,12 @@ __device__ __forceinline__ void add4(float* grad, const float* v) {
   }
 }
 
+// PROBE: the group that takes tile `fail` treats its second layer's wait there as given up, after it has
+// completed (kf_mlp_wait_probe: what a wait that gives up leaves in the outputs).
+template <bool PROBE>
 __global__ void __launch_bounds__(grd::kGroups* kGroup, 1)
     k_mlp_loss_grad(const float* __restrict__ params, const float* __restrict__ feats, const float* __restrict__ labels,
-                    int n, float inv_n, float* __restrict__ grad, float* __restrict__ loss) {
+                    int n, float inv_n, float* __restrict__ grad, float* __restrict__ loss, int fail) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned char* S = smem_raw + ((1024 - (tc::smem_u32(smem_raw) & 1023)) & 1023);
   const uint32_t sb = tc::smem_u32(S);
@@ -524,6 +527,7 @@ __global__ void __launch_bounds__(grd::kGroups* kGroup, 1)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(S + grd::TMEM);
   int* lock = reinterpret_cast<int*>(S + grd::LOCK);  // 1: the e tile is taken
   int* used = reinterpret_cast<int*>(S + grd::USED);  // 1: the gradient accumulators hold a tile
+  int* failed = reinterpret_cast<int*>(S + grd::FAILED);  // 1: a wait of the block gave up
   const int gi = threadIdx.x / kGroup, t = threadIdx.x % kGroup;
   const int warp = __shfl_sync(0xffffffffu, t >> 5, 0);  // (uniform, so that the MMAs' operands are too)
   const int row = t & (kTcM - 1), half = t / kTcM;
@@ -545,7 +549,7 @@ __global__ void __launch_bounds__(grd::kGroups* kGroup, 1)
     *reinterpret_cast<uint4*>(S + grd::E + tc::kmajor_off(i >> 3, 24 + (i & 7), grd::kEK)) = make_uint4(0u, 0u, 0u, 0u);
   const float b3 = params[kMlpB3];
   if (threadIdx.x < 32) tc::tmem_alloc(tmem_slot, grd::kCols);
-  if (threadIdx.x == 0) *lock = *used = 0;
+  if (threadIdx.x == 0) *lock = *used = *failed = 0;
   if (t == 0) {
     tc::mbar_init(bar, 1);
     tc::mbar_init(bar + 1, 1);
@@ -615,6 +619,7 @@ __global__ void __launch_bounds__(grd::kGroups* kGroup, 1)
     if (warp == 0 && tc::elect_one())
       mma_split_ta<true, grd::W2_T>(d + grd::kColD2, d, 0, kmajor<kMlpHid>(sb + grd::W2), id_kk, bar);
     ok = ok && tc::mbar_wait(bar, phase);
+    if (PROBE && tile == fail) ok = false;
     phase ^= 1u;
     tc::fence_after_sync();
     {  // logit from the two halves' partial sums
@@ -722,15 +727,15 @@ __global__ void __launch_bounds__(grd::kGroups* kGroup, 1)
     }
   }
   if (tc::bar_or(bid, kGroup, !ok)) {
-    // A tensor-core wait gave up: the loss becomes NaN; the MMAs in flight get one more bounded wait
-    // before the tensor memory is released.
+    // A tensor-core wait gave up: the loss becomes NaN and the block adds nothing to the gradient; the
+    // MMAs in flight get one more bounded wait before the tensor memory is released.
     if (t == 0) {
+      *failed = 1;
       if (locked) atomicExch(lock, 0);
       atomicAdd(loss, __int_as_float(0x7fc00000));
     }
     tc::mbar_wait(bar, phase ^ 1u);
     tc::mbar_wait(bar + 1, gphase ^ 1u);
-    gsum = lsum = 0.f;
   }
   // dW3, db3 and the loss: over the warp's samples, then over the eight warps of each half.
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -752,7 +757,7 @@ __global__ void __launch_bounds__(grd::kGroups* kGroup, 1)
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
-  if (threadIdx.x < kMlpHid + 2) {
+  if (threadIdx.x < kMlpHid + 2 && *failed == 0) {
     const int j = threadIdx.x;  // dW3[j], db3, loss: warps 0-3 and 8-11 hold units 0-31, the others 32-63
     float v = 0.f;
     for (int w = 0; w < 16; ++w) {
@@ -779,7 +784,7 @@ __global__ void __launch_bounds__(grd::kGroups* kGroup, 1)
 #pragma unroll
         for (int i = 0; i < 16; ++i) z[i] = (z[i] + m[i]) * inv_n;
     };
-    const bool any = *used != 0;
+    const bool any = *used != 0 && *failed == 0;
     if (any) {
       tc::tmem_ld16(tmem + lane_off + grd::kColG2 + 16 * q, v);
       tc::tmem_ld16(tmem + lane_off + grd::kColG2 + 64 + 16 * q, w);
@@ -843,12 +848,14 @@ __global__ void k_mlp_adam(float* params, const float* grad, float* m, float* v,
 // Number of SMs of the current device and, once per device, the kernel's shared-memory opt-in.
 static int tc_prepare(const void* kernel, int smem, int* sms) {
   static int sm_count[64] = {0};
-  static int smem_set[2][64] = {{0}};
+  static int smem_set[3][64] = {{0}};
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return -3;
   if (!sm_count[dev] && cudaDeviceGetAttribute(&sm_count[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return -3;
-  const int which = kernel == reinterpret_cast<const void*>(k_mlp_forward) ? 0 : 1;
+  const int which = kernel == reinterpret_cast<const void*>(k_mlp_forward)            ? 0
+                    : kernel == reinterpret_cast<const void*>(k_mlp_loss_grad<false>) ? 1
+                                                                                      : 2;
   if (smem > smem_set[which][dev]) {
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return -3;
     smem_set[which][dev] = smem;
@@ -867,17 +874,28 @@ int launch_mlp_forward(const float* params, const float* feats, int n, float* lo
   return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
-int launch_mlp_loss_grad(const float* params, const float* feats, const float* labels, int n, float* grad, float* loss,
-                         cudaStream_t st) {
+template <bool PROBE>
+static int launch_loss_grad(const float* params, const float* feats, const float* labels, int n, float* grad, float* loss,
+                            int fail, cudaStream_t st) {
   const int smem = static_cast<int>(grd::BYTES) + 1024;
   int sms = 0;
-  if (tc_prepare(reinterpret_cast<const void*>(k_mlp_loss_grad), smem, &sms) != 0) return -3;
+  if (tc_prepare(reinterpret_cast<const void*>(k_mlp_loss_grad<PROBE>), smem, &sms) != 0) return -3;
   launch_pdl(k_mlp_zero, (kMlpParams + 256) / 256, 256, 0, st, grad, loss);
   const int tiles = (n + kTcM - 1) / kTcM;
   if (n > 0)
-    launch_pdl(k_mlp_loss_grad, std::min(tiles, sms), grd::kGroups * kGroup, smem, st, params, feats, labels, n, 1.f / n, grad,
-               loss);
+    launch_pdl(k_mlp_loss_grad<PROBE>, std::min(tiles, sms), grd::kGroups * kGroup, smem, st, params, feats, labels, n, 1.f / n,
+               grad, loss, fail);
   return cudaGetLastError() == cudaSuccess ? 0 : -3;
+}
+
+int launch_mlp_loss_grad(const float* params, const float* feats, const float* labels, int n, float* grad, float* loss,
+                         cudaStream_t st) {
+  return launch_loss_grad<false>(params, feats, labels, n, grad, loss, -1, st);
+}
+
+int launch_mlp_wait_probe(const float* params, const float* feats, const float* labels, int n, float* grad, float* loss,
+                          int fail, cudaStream_t st) {
+  return launch_loss_grad<true>(params, feats, labels, n, grad, loss, fail, st);
 }
 
 int launch_mlp_adam(float* params, const float* grad, float* m, float* v, int t, float lr, float b1, float b2, float eps,

@@ -139,6 +139,8 @@ __device__ __forceinline__ float2 mlp_logit8(const uint4* __restrict__ frag, con
 }
 
 int launch_mlp_forward(const float* params, const float* feats, int n, float* logits, cudaStream_t st);
+int launch_mlp_wait_probe(const float* params, const float* feats, const float* labels, int n, float* grad, float* loss,
+                          int fail, cudaStream_t st);
 int launch_mlp_loss_grad(const float* params, const float* feats, const float* labels, int n, float* grad, float* loss,
                          cudaStream_t st);
 int launch_mlp_adam(float* params, const float* grad, float* m, float* v, int t, float lr, float b1, float b2, float eps,

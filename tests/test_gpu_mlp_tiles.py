@@ -75,3 +75,25 @@ def test_gradient_at_tile_edges(kf, n, shift):
     assert ((grad.double() - want).abs() <= 2.0 ** -15 * size).all()
     assert abs(loss.item() - (torch.nn.functional.softplus(z) - z * y).mean().item()) <= 1e-5
     assert (room[:shift] == 7.0).all() and (room[shift + kf.MLP_PARAMS:] == 7.0).all()
+
+
+# (a block's only tile; the first tiles of its two groups; a later one of the first)
+@pytest.mark.parametrize("n,tile", [(128, 0), (40000, 0), (40000, 200), (100003, 0), (100003, 200), (100003, 450)])
+def test_a_wait_that_gives_up_adds_nothing_of_its_block(kf, n, tile):
+    """The loss says so (NaN), and the gradient is that of the other blocks' tiles (block b takes the
+    tiles b, b + blocks, ...), none of the failed block's partial sums."""
+    params, rows, labels = _inputs(kf, n, n + 2)
+    blocks = min((n + 127) // 128, torch.cuda.get_device_properties(0).multi_processor_count)
+    loss, grad = kf.mlp_wait_probe(params, rows, labels, tile)
+    assert loss.isnan().all()
+    other = (torch.arange(n, device="cuda") // 128) % blocks != tile % blocks
+    W, x, h1, h2, z, _, _, _ = _net(params, rows[other])
+    g = torch.sigmoid(z) - labels[other].double()
+    e2 = g[:, None] * W[4] * (h2 > 0)
+    e1 = (e2 @ W[2]) * (h1 > 0)
+    want = torch.cat([(e1.T @ x).reshape(-1), e1.sum(0), (e2.T @ h1).reshape(-1), e2.sum(0), h2.T @ g, g.sum()[None]]) / n
+    # FP32 sums: about 1e-6 of the gradient's norm; one block's share is 1 / 152 of it
+    assert (grad.double() - want).norm() <= 2e-5 * want.norm() if other.any() else not grad.any()
+    # the call without a failure is whole again
+    loss, grad = kf.mlp_loss_grad(params, rows, labels)
+    assert loss.isfinite().all() and grad.isfinite().all()
