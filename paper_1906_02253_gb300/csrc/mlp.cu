@@ -96,14 +96,15 @@ __device__ __forceinline__ void stage_weights_b(const float* __restrict__ params
   }
 }
 
-// Raw features [8 h, 8 h + 8) of sample r (zeros past n and past the 14 inputs), loaded ahead of
-// their tile.
-__device__ __forceinline__ void fetch_half(const float* __restrict__ feats, int r, int n, int half, float2* f) {
+// Raw features [8 h, 8 h + 8) of sample r (zeros past the 14 inputs), loaded ahead of their tile.
+// Past n the features are the normaliser's mean (in shared memory).
+__device__ __forceinline__ void fetch_half(const float* __restrict__ feats, int r, int n, int half, const float* mean,
+                                           float2* f) {
   const float2* f2 = reinterpret_cast<const float2*>(feats + static_cast<size_t>(r) * kMlpIn);
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const int k = 4 * half + i;
-    f[i] = (r < n && k < kMlpIn / 2) ? __ldg(f2 + k) : make_float2(0.f, 0.f);
+    f[i] = r >= n ? reinterpret_cast<const float2*>(mean)[k] : k < kMlpIn / 2 ? __ldg(f2 + k) : make_float2(0.f, 0.f);
   }
 }
 
@@ -125,7 +126,9 @@ __device__ __forceinline__ bool stage_normaliser(const float* __restrict__ param
 
 // Standardised inputs [8 h, 8 h + 8), split for their tile. The quotient is a / sd from its
 // reciprocal with one correction by the remainder (divisions were a seventh of the forward pass's
-// instructions). Rows past n hold some finite value here: nothing of theirs is written or summed.
+// instructions). Rows past n hold zeros: the gradient MMAs multiply them by errors that are zero, so
+// they have to be finite whatever the normaliser is (as (0 - mean) / sd they were infinite for a large mean
+// over a small sd, and made the gradient NaN).
 __device__ __forceinline__ void standardise_half(const float2* f, int half, const float* mean, const float* sd,
                                                  const float* rs, bool by_reciprocal, uint4 (&x)[3]) {
   float v[8];
@@ -282,7 +285,7 @@ __global__ void __launch_bounds__(fwd::kGroups* kGroup, 1) k_mlp_forward(const f
   // during the second.
   float2 fin[4];
   uint4 x[3];
-  fetch_half(feats, tile * kTcM + row, n, half, fin);
+  fetch_half(feats, tile * kTcM + row, n, half, mean, fin);
   standardise_half(fin, half, mean, sd, rs, by_rs, x);
   for (; tile < n_tiles; tile += stride) {
     const int r = tile * kTcM + row;
@@ -291,7 +294,7 @@ __global__ void __launch_bounds__(fwd::kGroups* kGroup, 1) k_mlp_forward(const f
     tc::bar_sync(bid, kGroup);
     if (warp == 0 && tc::elect_one())
       mma_split16<fwd::X_T, fwd::W1_T>(d, kmajor<kTcK1>(sb + h_off), kmajor<kTcK1>(sb + fwd::W1), idesc, bar);
-    if (tile + stride < n_tiles) fetch_half(feats, (tile + stride) * kTcM + row, n, half, fin);
+    if (tile + stride < n_tiles) fetch_half(feats, (tile + stride) * kTcM + row, n, half, mean, fin);
     ok = ok && tc::mbar_wait(bar, phase);
     phase ^= 1u;
     tc::fence_after_sync();
@@ -578,7 +581,7 @@ __global__ void __launch_bounds__(grd::kGroups* kGroup, 1)
   // split during the gradient MMAs.
   float2 fin[4];
   uint4 x[3];
-  fetch_half(feats, tile * kTcM + row, n, half, fin);
+  fetch_half(feats, tile * kTcM + row, n, half, mean, fin);
   standardise_half(fin, half, mean, sd, rs, by_rs, x);
   float yin = tile * kTcM + row < n ? labels[tile * kTcM + row] : 0.f;
   for (; tile < n_tiles; tile += stride) {
@@ -686,7 +689,7 @@ __global__ void __launch_bounds__(grd::kGroups* kGroup, 1)
       mma_grad<64, grd::kHm, 144, grd::kHh, 80, grd::kHl, 64>(tmem + grd::kColG2, e_mn, xh_mn, bar + 1, *used != 0);
     if (tile + stride < n_tiles) {
       const int rn = (tile + stride) * kTcM + row;
-      fetch_half(feats, rn, n, half, fin);
+      fetch_half(feats, rn, n, half, mean, fin);
       yin = rn < n ? labels[rn] : 0.f;
     }
     if (half == 0) {  // under the gradient MMA

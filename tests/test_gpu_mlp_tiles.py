@@ -97,3 +97,23 @@ def test_a_wait_that_gives_up_adds_nothing_of_its_block(kf, n, tile):
     # the call without a failure is whole again
     loss, grad = kf.mlp_loss_grad(params, rows, labels)
     assert loss.isfinite().all() and grad.isfinite().all()
+
+
+@pytest.mark.parametrize("n", [1, 127, 129, 20000])
+@pytest.mark.parametrize("mean,sd", [(1e38, 0.1), (-1e38, 0.1), (1e5, 1e-35), (3.0, 1e-44)])
+def test_rows_past_the_end_leave_no_trace(kf, n, mean, sd):
+    """A constant feature at a mean far beyond its spread is zero in every row, whatever the normaliser
+    would make of a row of zeros."""
+    params, rows, labels = _inputs(kf, n, n + 3)
+    params[5185 + 3], params[5199 + 3] = mean, sd
+    rows[:, 3] = mean
+    loss, grad = kf.mlp_loss_grad(params, rows, labels)
+    out = kf.mlp_forward(params, rows)
+    params[5185 + 3], params[5199 + 3] = 0.0, 1.0
+    rows[:, 3] = 0.0
+    want_loss, want = kf.mlp_loss_grad(params, rows, labels)
+    # the same inputs but for the quotient's last bit; the blocks' sums are added in any order
+    assert grad.isfinite().all() and (grad - want).norm() <= 1e-5 * want.norm()
+    assert abs(loss.item() - want_loss.item()) <= 1e-5 * want_loss.item()
+    want = kf.mlp_forward(params, rows)
+    assert (out - want).abs().max() <= 1e-5 * want.abs().max().clamp(min=1.0)
