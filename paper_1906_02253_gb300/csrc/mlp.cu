@@ -96,15 +96,14 @@ __device__ __forceinline__ void stage_weights_b(const float* __restrict__ params
   }
 }
 
-// Raw features [8 h, 8 h + 8) of sample r (zeros past the 14 inputs), loaded ahead of their tile.
-// Past n the features are the normaliser's mean (in shared memory).
-__device__ __forceinline__ void fetch_half(const float* __restrict__ feats, int r, int n, int half, const float* mean,
-                                           float2* f) {
+// Raw features [8 h, 8 h + 8) of sample r (zeros past n and past the 14 inputs), loaded ahead of
+// their tile.
+__device__ __forceinline__ void fetch_half(const float* __restrict__ feats, int r, int n, int half, float2* f) {
   const float2* f2 = reinterpret_cast<const float2*>(feats + static_cast<size_t>(r) * kMlpIn);
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const int k = 4 * half + i;
-    f[i] = r >= n ? reinterpret_cast<const float2*>(mean)[k] : k < kMlpIn / 2 ? __ldg(f2 + k) : make_float2(0.f, 0.f);
+    f[i] = (r < n && k < kMlpIn / 2) ? __ldg(f2 + k) : make_float2(0.f, 0.f);
   }
 }
 
@@ -126,9 +125,9 @@ __device__ __forceinline__ bool stage_normaliser(const float* __restrict__ param
 
 // Standardised inputs [8 h, 8 h + 8), split for their tile. The quotient is a / sd from its
 // reciprocal with one correction by the remainder (divisions were a seventh of the forward pass's
-// instructions). Rows past n hold zeros: the gradient MMAs multiply them by errors that are zero, so
-// they have to be finite whatever the normaliser is (as (0 - mean) / sd they were infinite for a large mean
-// over a small sd, and made the gradient NaN).
+// instructions). A row past n, fetched as zeros, is (0 - mean) / sd in the forward pass, where it meets
+// nothing else; in the loss gradient, whose MMAs multiply it by an error of zero, it has to be finite
+// whatever the normaliser is, and a mean of zeros is passed for it.
 __device__ __forceinline__ void standardise_half(const float2* f, int half, const float* mean, const float* sd,
                                                  const float* rs, bool by_reciprocal, uint4 (&x)[3]) {
   float v[8];
@@ -285,7 +284,7 @@ __global__ void __launch_bounds__(fwd::kGroups* kGroup, 1) k_mlp_forward(const f
   // during the second.
   float2 fin[4];
   uint4 x[3];
-  fetch_half(feats, tile * kTcM + row, n, half, mean, fin);
+  fetch_half(feats, tile * kTcM + row, n, half, fin);
   standardise_half(fin, half, mean, sd, rs, by_rs, x);
   for (; tile < n_tiles; tile += stride) {
     const int r = tile * kTcM + row;
@@ -294,7 +293,7 @@ __global__ void __launch_bounds__(fwd::kGroups* kGroup, 1) k_mlp_forward(const f
     tc::bar_sync(bid, kGroup);
     if (warp == 0 && tc::elect_one())
       mma_split16<fwd::X_T, fwd::W1_T>(d, kmajor<kTcK1>(sb + h_off), kmajor<kTcK1>(sb + fwd::W1), idesc, bar);
-    if (tile + stride < n_tiles) fetch_half(feats, (tile + stride) * kTcM + row, n, half, mean, fin);
+    if (tile + stride < n_tiles) fetch_half(feats, (tile + stride) * kTcM + row, n, half, fin);
     ok = ok && tc::mbar_wait(bar, phase);
     phase ^= 1u;
     tc::fence_after_sync();
@@ -462,7 +461,7 @@ constexpr int kXhK = 240, kEK = 256;                            // columns of th
 constexpr int kHm = 0, kHh = 8, kXh = 16, kXm = 18, kXl = 20, kHl = 22;  // 8-column blocks of the parts
 constexpr uint32_t E_T = kTcM * kEK * 2, XH_T = kTcM * kXhK * 2, W1_T = 2048, W2_T = 8192;  // bytes of one tile
 constexpr uint32_t E = 0, XH = E + E_T, W2 = XH + kGroups * XH_T, W1 = W2 + 3 * W2_T, B2 = W1 + 3 * W1_T,
-                   W3 = B2 + 256, MEAN = W3 + 256, SD = MEAN + 64, RS = SD + 64, PART = RS + 64, RED = PART + kGroups * 1024,
+                   W3 = B2 + 256, MEAN = W3 + 256, SD = MEAN + 64, RS = SD + 64, NIL = RS + 64, PART = NIL + 64, RED = PART + kGroups * 1024,
                    BAR = RED + 16 * 34 * 4, TMEM = BAR + 16 * kGroups, LOCK = TMEM + 4, USED = LOCK + 4, FAILED = USED + 4, BYTES = FAILED + 8;
 static_assert(BYTES + 1024 <= 227 * 1024, "shared-memory layout");
 constexpr uint32_t kCols = 512, kColD2 = 96, kColG2 = 320, kColG1 = 464;
@@ -526,6 +525,7 @@ __global__ void __launch_bounds__(grd::kGroups* kGroup, 1)
   float* mean = reinterpret_cast<float*>(S + grd::MEAN);
   float* sd = reinterpret_cast<float*>(S + grd::SD);
   float* rs = reinterpret_cast<float*>(S + grd::RS);
+  float* nil = reinterpret_cast<float*>(S + grd::NIL);  // [16] zeros
   float* red = reinterpret_cast<float*>(S + grd::RED);  // [16 warps][34]: dW3 of the warp's 32 units, db3, loss
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(S + grd::TMEM);
   int* lock = reinterpret_cast<int*>(S + grd::LOCK);  // 1: the e tile is taken
@@ -548,6 +548,7 @@ __global__ void __launch_bounds__(grd::kGroups* kGroup, 1)
     w3[threadIdx.x] = params[kMlpW3 + threadIdx.x];
   }
   const bool odd_sd = !stage_normaliser(params, mean, sd, rs);
+  if (threadIdx.x < kTcK1) nil[threadIdx.x] = 0.f;
   for (int i = threadIdx.x; i < kTcM * 8; i += blockDim.x)  // the e tile's zero columns
     *reinterpret_cast<uint4*>(S + grd::E + tc::kmajor_off(i >> 3, 24 + (i & 7), grd::kEK)) = make_uint4(0u, 0u, 0u, 0u);
   const float b3 = params[kMlpB3];
@@ -581,8 +582,8 @@ __global__ void __launch_bounds__(grd::kGroups* kGroup, 1)
   // split during the gradient MMAs.
   float2 fin[4];
   uint4 x[3];
-  fetch_half(feats, tile * kTcM + row, n, half, mean, fin);
-  standardise_half(fin, half, mean, sd, rs, by_rs, x);
+  fetch_half(feats, tile * kTcM + row, n, half, fin);
+  standardise_half(fin, half, tile * kTcM + row < n ? mean : nil, sd, rs, by_rs, x);
   float yin = tile * kTcM + row < n ? labels[tile * kTcM + row] : 0.f;
   for (; tile < n_tiles; tile += stride) {
     const bool valid = tile * kTcM + row < n;
@@ -689,7 +690,7 @@ __global__ void __launch_bounds__(grd::kGroups* kGroup, 1)
       mma_grad<64, grd::kHm, 144, grd::kHh, 80, grd::kHl, 64>(tmem + grd::kColG2, e_mn, xh_mn, bar + 1, *used != 0);
     if (tile + stride < n_tiles) {
       const int rn = (tile + stride) * kTcM + row;
-      fetch_half(feats, rn, n, half, mean, fin);
+      fetch_half(feats, rn, n, half, fin);
       yin = rn < n ? labels[rn] : 0.f;
     }
     if (half == 0) {  // under the gradient MMA
@@ -718,7 +719,7 @@ __global__ void __launch_bounds__(grd::kGroups* kGroup, 1)
     // Dg1 += E1^T X
     if (warp == 0 && tc::elect_one())
       mma_grad<0, grd::kXh, 32, grd::kXh, 16, grd::kXl, 16>(tmem + grd::kColG1, e_mn, xh_mn, bar + 1, *used != 0);
-    standardise_half(fin, half, mean, sd, rs, by_rs, x);
+    standardise_half(fin, half, (tile + stride) * kTcM + row < n ? mean : nil, sd, rs, by_rs, x);
     ok = ok && tc::mbar_wait(bar + 1, gphase);
     gphase ^= 1u;
     tc::fence_after_sync();
