@@ -462,7 +462,7 @@ constexpr int kHm = 0, kHh = 8, kXh = 16, kXm = 18, kXl = 20, kHl = 22;  // 8-co
 constexpr uint32_t E_T = kTcM * kEK * 2, XH_T = kTcM * kXhK * 2, W1_T = 2048, W2_T = 8192;  // bytes of one tile
 constexpr uint32_t E = 0, XH = E + E_T, W2 = XH + kGroups * XH_T, W1 = W2 + 3 * W2_T, B2 = W1 + 3 * W1_T,
                    W3 = B2 + 256, MEAN = W3 + 256, SD = MEAN + 64, RS = SD + 64, NIL = RS + 64, PART = NIL + 64, RED = PART + kGroups * 1024,
-                   BAR = RED + 16 * 34 * 4, TMEM = BAR + 16 * kGroups, LOCK = TMEM + 4, USED = LOCK + 4, FAILED = USED + 4, BYTES = FAILED + 8;
+                   BAR = RED + 16 * 34 * 4, TMEM = BAR + 16 * kGroups, LOCK = TMEM + 4, USED = LOCK + 4, BYTES = USED + 8;
 static_assert(BYTES + 1024 <= 227 * 1024, "shared-memory layout");
 constexpr uint32_t kCols = 512, kColD2 = 96, kColG2 = 320, kColG1 = 464;
 }  // namespace grd
@@ -530,7 +530,6 @@ __global__ void __launch_bounds__(grd::kGroups* kGroup, 1)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(S + grd::TMEM);
   int* lock = reinterpret_cast<int*>(S + grd::LOCK);  // 1: the e tile is taken
   int* used = reinterpret_cast<int*>(S + grd::USED);  // 1: the gradient accumulators hold a tile
-  int* failed = reinterpret_cast<int*>(S + grd::FAILED);  // 1: a wait of the block gave up
   const int gi = threadIdx.x / kGroup, t = threadIdx.x % kGroup;
   const int warp = __shfl_sync(0xffffffffu, t >> 5, 0);  // (uniform, so that the MMAs' operands are too)
   const int row = t & (kTcM - 1), half = t / kTcM;
@@ -553,7 +552,7 @@ __global__ void __launch_bounds__(grd::kGroups* kGroup, 1)
     *reinterpret_cast<uint4*>(S + grd::E + tc::kmajor_off(i >> 3, 24 + (i & 7), grd::kEK)) = make_uint4(0u, 0u, 0u, 0u);
   const float b3 = params[kMlpB3];
   if (threadIdx.x < 32) tc::tmem_alloc(tmem_slot, grd::kCols);
-  if (threadIdx.x == 0) *lock = *used = *failed = 0;
+  if (threadIdx.x == 0) *lock = *used = 0;
   if (t == 0) {
     tc::mbar_init(bar, 1);
     tc::mbar_init(bar + 1, 1);
@@ -734,12 +733,12 @@ __global__ void __launch_bounds__(grd::kGroups* kGroup, 1)
     // A tensor-core wait gave up: the loss becomes NaN and the block adds nothing to the gradient; the
     // MMAs in flight get one more bounded wait before the tensor memory is released.
     if (t == 0) {
-      *failed = 1;
       if (locked) atomicExch(lock, 0);
       atomicAdd(loss, __int_as_float(0x7fc00000));
     }
     tc::mbar_wait(bar, phase ^ 1u);
     tc::mbar_wait(bar + 1, gphase ^ 1u);
+    gsum = lsum = 0.f;
   }
   // dW3, db3 and the loss: over the warp's samples, then over the eight warps of each half.
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -759,9 +758,9 @@ __global__ void __launch_bounds__(grd::kGroups* kGroup, 1)
     red[wid * 34 + 33] = lsum;
   }
   tc::fence_before_sync();
-  __syncthreads();
+  const bool failed = __syncthreads_or(!ok);
   tc::fence_after_sync();
-  if (threadIdx.x < kMlpHid + 2 && *failed == 0) {
+  if (threadIdx.x < kMlpHid + 2 && !failed) {
     const int j = threadIdx.x;  // dW3[j], db3, loss: warps 0-3 and 8-11 hold units 0-31, the others 32-63
     float v = 0.f;
     for (int w = 0; w < 16; ++w) {
@@ -788,7 +787,7 @@ __global__ void __launch_bounds__(grd::kGroups* kGroup, 1)
 #pragma unroll
         for (int i = 0; i < 16; ++i) z[i] = (z[i] + m[i]) * inv_n;
     };
-    const bool any = *used != 0 && *failed == 0;
+    const bool any = *used != 0 && !failed;
     if (any) {
       tc::tmem_ld16(tmem + lane_off + grd::kColG2 + 16 * q, v);
       tc::tmem_ld16(tmem + lane_off + grd::kColG2 + 64 + 16 * q, w);
