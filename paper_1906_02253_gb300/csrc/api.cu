@@ -484,8 +484,9 @@ int kf_autotune_find(const KfGeometry* geom, const KfHitIndex* index, const floa
   for (int c : caps)
     if (c >= need && n_cap < 2) cap_opts[n_cap++] = c;
   // With k_max > 4 adaptive capacities 2 and 4 are tried too, those that hold top_n with the
-  // learned proposal (a configuration whose workspace does not fit the caller's fails and is
-  // passed over).
+  // learned proposal and whose whole workspace, overflow list and seed order, fits the caller's: one
+  // sized for a single pass has room for either, and would set two passes without the order
+  // against single passes with it.
   const bool learned = params->mlp && params->top_n > 0;
   int ad_opts[3] = {0, 0, 0}, n_ad = 1;
   if (params->k_max > 4)
@@ -501,6 +502,7 @@ int kf_autotune_find(const KfGeometry* geom, const KfHitIndex* index, const floa
         p.k_capacity = cap_opts[ci2];
         p.blocks_per_sm = 0;
         p.adaptive_capacity = ad_opts[ai];
+        if (ad_opts[ai] > 0 && workspace_bytes < kf_find_workspace_size(n_seeds, &p)) continue;
         const float t = time_config(st, [&]() {
           return kf_find_tracks(geom, index, hits, hit_surface, seed_hits, seed_event, n_seeds, &p, hits_out,
                                 nhits_out, chi2_out, state_out, cov_out, status_out, workspace, workspace_bytes, stream);

@@ -521,6 +521,29 @@ def test_autotuner_configurations_give_identical_results(kf):
     assert blk in range(64, 257, 32) and ms > 0
 
 
+def test_autotuner_compares_launches_of_whole_workspaces(kf):
+    """A workspace sized for a single pass holds its seed order or two passes' overflow list, not both:
+    two passes are left out there, also where they would be faster even without the order."""
+    import ctypes
+    wl = synth.workload("find", n_events=10)
+    b = synth.generate(wl)
+    g = kf.Geometry(wl)
+    dev = kf.to_device_event_batch(b)
+    idx = kf.build_hit_index(g, dev["hits"], dev["slab_offsets"], b.n_events, dev["max_slab_hits"])
+    prm = kf.find_params(wl.chi2_cut, 16, wl.max_miss, wl.lmax)
+    n = dev["seed_hits"].shape[1]
+    out = kf.find_tracks(g, idx, dev["hits"], dev["hit_surface"], dev["seed_hits"], dev["seed_event"], prm)
+    P = lambda t: ctypes.c_void_p(t.data_ptr())  # noqa: E731
+    room = torch.empty(kf.find_workspace_size(n, prm), dtype=torch.uint8, device="cuda")
+    ms = ctypes.c_float()
+    rc = kf.load_library().kf_autotune_find(
+        g.ref, ctypes.byref(idx.c), P(dev["hits"]), P(dev["hit_surface"]), P(dev["seed_hits"]), P(dev["seed_event"]), n,
+        ctypes.byref(prm), P(out["hits"]), P(out["nhits"]), P(out["chi2"]), P(out["state"]), P(out["cov"]), P(out["status"]),
+        P(room), room.numel(), ctypes.byref(ms), ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+    assert rc == kf.KF_OK and ms.value > 0
+    assert prm.adaptive_capacity == 0
+
+
 def _find_gpu(kf, wl, b, **kw):
     g = kf.Geometry(wl)
     dev = kf.to_device_event_batch(b)
