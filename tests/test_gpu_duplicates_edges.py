@@ -1,5 +1,6 @@
-"""Duplicate removal counts shared hits through the hits' users: lists with hits at or above n_hits
-(which the inverted index leaves out but the lists share), the same hit twice in a list, empty
+"""Duplicate removal counts shared hits through the hits' users, or through the lists where a hit has
+many: hits with fewer and with more users than twice a list's entries, lists with hits at or above
+n_hits (which the inverted index leaves out but the lists share), the same hit twice in a list, empty
 lists, equal chi2 and directions at the cut, against a pass over all pairs."""
 import numpy as np
 import pytest
@@ -9,7 +10,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("n,lmax,n_hits,top", [(1, 1, 1, 1), (40, 4, 12, 12), (400, 17, 300, 300), (400, 31, 200, 260),
-                                               (129, 5, 0, 9)])
+                                               (129, 5, 0, 9), (600, 9, 250, 270), (500, 6, 9, 11)])
 def test_all_pairs(n, lmax, n_hits, top):
     import __graft_entry__ as ge
     ge.build_library()
