@@ -18,7 +18,6 @@ __global__ void k_build_hit_index(DevGeom G, const float2* hits, const int* slab
 __global__ void k_build_hit_index_fine(const __grid_constant__ DevGeom G, const float2* hits, const int* slab_off,
                                        int n_slabs, int cap, int* bin_off, float2* sorted_hits, int* sorted_ids,
                                        float4* sorted_rec, uint4* sub_off, int* d_status);
-constexpr int kFineMaxBins = 8192;  // hitindex.cu
 __global__ void k_fit_tracks(DevGeom G, const __grid_constant__ DevMat M, const float2* hits, const int* hit_surface,
                              const int* track_hits,
                              int n_tracks, int lmax, float* state_out, float* cov_out, float* chi2_out, int* ndof_out,
@@ -236,7 +235,10 @@ int kf_build_hit_index(const KfGeometry* geom, const float* hits, const int* sla
   // and 5 a hit of shared memory instead of 16 and 4.
   const size_t by_bins = static_cast<size_t>(G.n_bins + 1) * sizeof(int) + 5 * static_cast<size_t>(cap);
   const size_t by_fine = static_cast<size_t>(G.n_bins) * 16 + 4 * static_cast<size_t>(cap);
-  constexpr size_t kHalf = 113 * 1024, kAll = 226 * 1024;
+  // (dynamic shared memory of a block when two share an SM's 228 KB, 1 KB of each block's reserved and
+  // 128 bytes static; of one alone in its 227 KB)
+  constexpr size_t kStatic = 32 * sizeof(int), kHalf = 113 * 1024 - kStatic, kAll = 226 * 1024;
+  static_assert(2 * (kHalf + kStatic + 1024) <= 228 * 1024 && kAll + kStatic <= 227 * 1024, "shared memory of an SM");
   const bool fine = G.n_bins <= kFineMaxBins && (by_fine <= kHalf || (by_bins > kHalf && by_fine <= kAll));
   const size_t smem = fine ? by_fine : by_bins;
   // Raise the kernel's dynamic shared memory limit once per device (and only when a larger slab

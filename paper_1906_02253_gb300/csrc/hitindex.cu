@@ -193,9 +193,6 @@ __global__ void __launch_bounds__(1024, 2) k_build_hit_index(DevGeom G, const fl
 // with bins and sub-bins apart, the search records 55 us of it; issue and latency bound (a slab is a
 // chain of eight block barriers). 512 or 768 threads a block are 2-3% slower, as the largest slab's
 // shared memory keeps it at two blocks per SM.
-constexpr int kFineMaxBins = 8192;
-static_assert(kFineMaxBins * kPhiSub <= 65536, "a fine bin is a 16-bit word");
-
 // 16-bit fields of x added up within the word pair by pair: (lo, lo + hi), plus c in both fields.
 __device__ __forceinline__ unsigned cumulate(unsigned x, unsigned c) { return x + (x << 16) + c * 0x10001u; }
 

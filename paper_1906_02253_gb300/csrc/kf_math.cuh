@@ -20,6 +20,8 @@ constexpr float kPiF = 3.14159265358979323846f;
 constexpr float kTwoPiF = 6.28318530717958647692f;
 constexpr float kCurvF = 0.00299792458f;  // GeV / (T cm)
 constexpr int kPhiSub = 8;                 // phi sub-bins per phi bin (KF_PHI_SUB)
+constexpr int kFineMaxBins = 8192;         // bins of a surface up to which a fine bin (bin * kPhiSub + sub-bin) is 16 bits
+static_assert(kFineMaxBins * kPhiSub <= 65536, "a fine bin is a 16-bit word");
 constexpr int kRegions = 5;                // tracking regions of the steering (KF_N_REGIONS)
 
 // Geometry as the kernels see it: passed by value, so it lives in the constant bank.

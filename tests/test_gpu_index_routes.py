@@ -40,7 +40,7 @@ def _reference(hits, n_phi, n_2nd):
 
 
 @pytest.mark.parametrize("n_phi,n_2nd", [(1, 1), (3, 5), (64, 32), (256, 32), (1024, 8), (257, 32), (128, 128)])
-@pytest.mark.parametrize("slabs", [(0, 1, 5, 0), (1000, 33, 20000), (32768, 3)])
+@pytest.mark.parametrize("slabs", [(0, 1, 5, 0), (1000, 33, 20000), (20704, 3), (20706, 3), (32768, 3)])  # (20,706 at 64 x 32 bins: two blocks of the fine kernel no longer fit an SM)
 def test_routes_match_the_bin_rule(kf, n_phi, n_2nd, slabs):
     surf = [SimpleNamespace(type=0, r_or_z=4.0 + i, lo=LO, hi=HI, x_over_x0=0.0, n_phi=n_phi, n_2nd=n_2nd)
             for i in range(len(slabs))]
