@@ -443,14 +443,6 @@ __device__ __forceinline__ bool load_seed(WarpSmem<KC>& W, int gbase, int slot, 
         make_float4(__int_as_float(3), __int_as_float(0), __int_as_float(0), __int_as_float(surf_word));
   return true;
 }
-// The same out of line, for the small plain instances and the steering ones: inlined there it makes
-// the compiler round one of the step's sums differently from the other instances, and an adaptive
-// capacity's two instances have to agree bit for bit (a test holds them to it). Elsewhere inlining
-// is faster (learned finding by 6%).
-template <int KC>
-__device__ __noinline__ bool load_seed_call(WarpSmem<KC>& W, int gbase, int slot, const float* rec, int surf_word) {
-  return load_seed(W, gbase, slot, rec, surf_word);
-}
 
 // Seed number s of the order that takes the front list's seeds first and the others, which that list
 // has not marked (nor as removed or failed), in index order. Out of line: once per seed.
@@ -609,8 +601,7 @@ __global__ void __launch_bounds__(LEARNED ? kFindMaxBlockLearned : 256, 2) k_fin
       }
       const float* rec = A.seed_state + static_cast<size_t>(seed) * kSeedWords;
       const int surf_word = STEER ? ((pos + 1) << 8) | (s3 & 255) : s3;
-      if constexpr (!LEARNED && (KC <= 4 || FEAT == kFeatSteer)) valid = load_seed_call(W, gbase, slot, rec, surf_word);
-      else valid = load_seed(W, gbase, slot, rec, surf_word);
+      valid = load_seed(W, gbase, slot, rec, surf_word);
       if (!valid) seed = -1;  // a failed seed's outputs were written by the seed-state kernel
       valid = valid && slot == 0;
     }

@@ -266,7 +266,10 @@ __device__ __forceinline__ bool apply_propagation(const DevGeom& G, const DevMat
   const float cot = ct / st;
   const float dx = s * (pr.c0 * pr.f1 - pr.s0 * pr.f2);
   const float dy = s * (pr.s0 * pr.f1 + pr.c0 * pr.f2);
-  const float cD = 1.f - 2.f * pr.sh * pr.sh, sD = 2.f * pr.sh * pr.ch;
+  // The cosine's product and difference are one fused operation, written out: the compiler rounded the
+  // product apart in some kernels and not in others (visible in 1 of 7,000 steps, in the covariance), and
+  // the finder's capacities have to agree bit for bit.
+  const float cD = fmaf(-2.f * pr.sh, pr.sh, 1.f), sD = 2.f * pr.sh * pr.ch;
   float d1, d2;
   helix_dfd(D, pr.f1, pr.q, cD, d1, d2);
   // Jacobian at fixed s.
