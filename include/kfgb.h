@@ -421,6 +421,7 @@ int kf_fp32_fma_probe(float* sink, int blocks, int iters, long long* flops, kf_s
 #define KF_PROBE_SINCOS 0
 #define KF_PROBE_ATAN_SMALL 1
 #define KF_PROBE_HALF_ANGLE 2
+#define KF_PROBE_WINDOW_AZIMUTH 3
 int kf_math_probe(int fn, const float* a, const float* b, int n, float* o0, float* o1, float* o2, kf_stream_t stream);
 
 /* Probe of the bounded wait that the tensor-core kernels use for MMA completion (measurement only,

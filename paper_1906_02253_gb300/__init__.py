@@ -354,7 +354,7 @@ def fp32_fma_rate(blocks: int = 0, iters: int = 4096, reps: int = 3, stream=None
     return best
 
 
-PROBE_SINCOS, PROBE_ATAN_SMALL, PROBE_HALF_ANGLE = 0, 1, 2  # KF_PROBE_*
+PROBE_SINCOS, PROBE_ATAN_SMALL, PROBE_HALF_ANGLE, PROBE_WINDOW_AZIMUTH = 0, 1, 2, 3  # KF_PROBE_*
 
 
 def wait_probe(limit_us: int, stream=None):
@@ -378,7 +378,7 @@ def mlp_wait_probe(params, features, labels, tile: int, stream=None):
 
 def math_probe(fn: int, a, b=None, stream=None):
     """kf_math_probe: the path's hand-written trigonometry on FP32 CUDA tensors a (and b for the
-    small-angle arctangent). Returns three tensors (o0, o1, o2) of a's shape."""
+    small-angle arctangent and the window's azimuth). Returns three tensors (o0, o1, o2) of a's shape."""
     lib = load_library()
     a = _cuda(a, torch.float32, "a").contiguous()
     b = None if b is None else _cuda(b, torch.float32, "b").contiguous()

@@ -585,9 +585,9 @@ int kf_fp32_fma_probe(float* sink, int blocks, int iters, long long* flops, kf_s
 }
 
 int kf_math_probe(int fn, const float* a, const float* b, int n, float* o0, float* o1, float* o2, kf_stream_t stream) {
-  if (fn < KF_PROBE_SINCOS || fn > KF_PROBE_HALF_ANGLE || n < 0) return KF_ERR_ARG;
+  if (fn < KF_PROBE_SINCOS || fn > KF_PROBE_WINDOW_AZIMUTH || n < 0) return KF_ERR_ARG;
   if (n == 0) return KF_OK;
-  if (!a || !o0 || !o1 || !o2 || (fn == KF_PROBE_ATAN_SMALL && !b)) return KF_ERR_ARG;
+  if (!a || !o0 || !o1 || !o2 || ((fn == KF_PROBE_ATAN_SMALL || fn == KF_PROBE_WINDOW_AZIMUTH) && !b)) return KF_ERR_ARG;
   return launch_math_probe(fn, a, b, n, o0, o1, o2, reinterpret_cast<cudaStream_t>(stream));
 }
 

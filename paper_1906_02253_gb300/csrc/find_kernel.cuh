@@ -208,25 +208,6 @@ __device__ __forceinline__ float resid_angle(float x, float y, float c, float s)
   return atan2_cold(a, b);
 }
 
-// Azimuth of (x, y), within 1e-6 rad: the arctangent's polynomial 4.4.49 of Abramowitz and Stegun,
-// Handbook of Mathematical Functions (error 2e-8 on [0, 1]), and the octants. For the search
-// window's centre, whose range is padded by 1e-5 rad; atan2f there cost 0.5% of the finder.
-__device__ __forceinline__ float window_azimuth(float x, float y) {
-  const float ax = fabsf(x), ay = fabsf(y), t = fminf(ax, ay) / fmaxf(ax, ay), t2 = t * t;
-  float r = 0.0028662257f;
-  r = fmaf(r, t2, -0.0161657367f);
-  r = fmaf(r, t2, 0.0429096138f);
-  r = fmaf(r, t2, -0.0752896400f);
-  r = fmaf(r, t2, 0.1065626393f);
-  r = fmaf(r, t2, -0.1420889944f);
-  r = fmaf(r, t2, 0.1999355085f);
-  r = fmaf(r, t2, -0.3333314528f);
-  r = fmaf(r * t2, t, t);
-  if (ay > ax) r = 0.5f * kPiF - r;
-  if (x < 0.f) r = kPiF - r;
-  return y < 0.f ? -r : r;
-}
-
 // chi2 of a hit's search record against a window (wa: x, y, centre of the 2nd coordinate,
 // transverse scale R; wb: S^-1 00, 01, 11 and the far-hit threshold t). With a = rho sin(dphi),
 // b = rho cos(dphi) (rho the predicted transverse radius), chi2 >= R^2 dphi^2 / S_00 >=

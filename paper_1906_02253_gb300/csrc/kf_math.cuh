@@ -100,6 +100,25 @@ __device__ __forceinline__ float atan_small(float a, float b) {
   return t * (1.f + t2 * (-1.f / 3.f + t2 * (1.f / 5.f + t2 * (-1.f / 7.f))));
 }
 
+// Azimuth of (x, y), within 1e-6 rad: the arctangent's polynomial 4.4.49 of Abramowitz and Stegun,
+// Handbook of Mathematical Functions (error 2e-8 on [0, 1]), and the octants. For the search
+// window's centre, whose range is padded by 1e-5 rad; atan2f there cost 0.5% of the finder.
+__device__ __forceinline__ float window_azimuth(float x, float y) {
+  const float ax = fabsf(x), ay = fabsf(y), t = fminf(ax, ay) / fmaxf(ax, ay), t2 = t * t;
+  float r = 0.0028662257f;
+  r = fmaf(r, t2, -0.0161657367f);
+  r = fmaf(r, t2, 0.0429096138f);
+  r = fmaf(r, t2, -0.0752896400f);
+  r = fmaf(r, t2, 0.1065626393f);
+  r = fmaf(r, t2, -0.1420889944f);
+  r = fmaf(r, t2, 0.1999355085f);
+  r = fmaf(r, t2, -0.3333314528f);
+  r = fmaf(r * t2, t, t);
+  if (ay > ax) r = 0.5f * kPiF - r;
+  if (x < 0.f) r = kPiF - r;
+  return y < 0.f ? -r : r;
+}
+
 // sin(D/2), cos(D/2) and q = sin(D/2)/(D/2); then f1 = sin(D)/D = q cos(D/2) and
 // f2 = (1 - cos D)/D = q sin(D/2).
 // Below |D/2| = 0.1 (every step of a track above ~0.1 GeV over a few cm) the Taylor series are

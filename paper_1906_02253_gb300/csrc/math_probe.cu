@@ -1,6 +1,6 @@
 // Accuracy probe of the hand-written trigonometry on the Kalman path (measurement only, not on
-// the path): evaluates sincos_small, atan_small and half_angle on caller-given arguments with the
-// same code and compiler flags as the finder and the fit, so that a test can compare them with
+// the path): evaluates sincos_small, atan_small, half_angle and window_azimuth on caller-given arguments
+// with the same code and compiler flags as the finder and the fit, so that a test can compare them with
 // the CUDA library's functions and with FP64 values.
 #include "../../include/kfgb.h"
 #include "kf_math.cuh"
@@ -15,6 +15,8 @@ __global__ void k_math_probe(int fn, const float* __restrict__ a, const float* _
       sincos_small(a[i], r0, r1);
     } else if (fn == KF_PROBE_ATAN_SMALL) {
       r0 = atan_small(a[i], b[i]);
+    } else if (fn == KF_PROBE_WINDOW_AZIMUTH) {
+      r0 = window_azimuth(a[i], b[i]);
     } else {
       half_angle(a[i], r0, r1, r2);
     }

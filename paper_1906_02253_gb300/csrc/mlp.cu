@@ -123,9 +123,11 @@ __device__ __forceinline__ bool stage_normaliser(const float* __restrict__ param
   return in_range;
 }
 
-// Standardised inputs [8 h, 8 h + 8), split for their tile. The quotient is a / sd from its
-// reciprocal with one correction by the remainder (divisions were a seventh of the forward pass's
-// instructions). A row past n, fetched as zeros, is (0 - mean) / sd in the forward pass, where it meets
+// Standardised inputs [8 h, 8 h + 8), split for their tile. The quotient is a / sd from the correctly
+// rounded reciprocal r: q = a r, then q + (a - q sd) r with the remainder exact in a fused operation
+// (P. W. Markstein, Computation of elementary functions on the IBM RISC System/6000 processor, IBM J.
+// Res. Dev. 34, 1990), the bits of the division (a test compares them); divisions were a seventh of the
+// forward pass's instructions. A row past n, fetched as zeros, is (0 - mean) / sd in the forward pass, where it meets
 // nothing else; in the loss gradient, whose MMAs multiply it by an error of zero, it has to be finite
 // whatever the normaliser is, and a mean of zeros is passed for it.
 __device__ __forceinline__ void standardise_half(const float2* f, int half, const float* mean, const float* sd,

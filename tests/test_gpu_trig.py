@@ -96,6 +96,26 @@ def test_half_angle_accuracy(kf):
     assert es.max() <= 2.0 and ec.max() <= 2.0
 
 
+def test_window_azimuth_accuracy(kf):
+    """The search window's centre, against the FP64 azimuth of the same FP32 point: all octants, the axes
+    and diagonals, radii from 0.01 to 1000 cm. The window's padding of 1e-5 rad takes the 1e-6 rad stated
+    for it (2e-8 of the polynomial, a fast-math quotient and the FP32 angle's own spacing, 2.4e-7 at pi)."""
+    rng = np.random.default_rng(8)
+    n = 1 << 21
+    t = np.concatenate([np.linspace(-np.pi, np.pi, n // 2), rng.uniform(-np.pi, np.pi, n // 2)])
+    r = 10.0 ** rng.uniform(-2, 3, n)
+    x, y = (r * np.cos(t)).astype(np.float32), (r * np.sin(t)).astype(np.float32)
+    e = np.float32([1.0, -1.0, 0.0, -0.0])
+    ax, ay = np.meshgrid(e, e)
+    keep = (ax != 0) | (ay != 0)
+    x, y = np.concatenate([x, ax[keep]]), np.concatenate([y, ay[keep]])
+    o, _, _ = kf.math_probe(kf.PROBE_WINDOW_AZIMUTH, torch.from_numpy(x).cuda(), torch.from_numpy(y).cuda())
+    d = o.cpu().numpy().astype(np.float64) - np.arctan2(y.astype(np.float64), x.astype(np.float64))
+    d = np.abs(np.remainder(d + np.pi, 2 * np.pi) - np.pi)  # (pi and -pi are the same direction)
+    print(f"largest error {d.max():.2e} rad")
+    assert d.max() <= 1e-6, (d.max(), x[d.argmax()], y[d.argmax()])
+
+
 def test_probe_rejects_bad_arguments(kf):
     lib = kf.load_library()
     assert lib.kf_math_probe(7, None, None, 1, None, None, None, None) == kf.KF_ERR_ARG
