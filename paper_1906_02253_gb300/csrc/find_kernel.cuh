@@ -520,6 +520,7 @@ __global__ void __launch_bounds__(LEARNED ? kFindMaxBlockLearned : 256, 2) k_fin
   // exactly its children.
   const int keep = LEARNED ? A.top_n : (A.detect ? min(A.k_max, KC) : A.k_max);
   const bool detect = A.detect != 0;
+  const bool beyond = detect && A.k_max > KC;  // passing hits beyond the lists count
   const bool margin_on = LEARNED && A.score_margin > 0.f;
   const bool window_rank = LEARNED && A.window_rank != 0;  // rank the window's box before the cut
   const int grp = lane / KC, slot = lane % KC;
@@ -543,7 +544,7 @@ __global__ void __launch_bounds__(LEARNED ? kFindMaxBlockLearned : 256, 2) k_fin
     // here rather than costing the group a step each.
     if (want && slot == 0) {
       s = atomicAdd(A.counter, 1);
-      if (A.seed_list)  // second pass of adaptive capacity: the first pass's overflowing seeds
+      if (A.seed_list)  // the list by direction, or (second pass) the first pass's overflowing seeds
         s = s < min(*A.seed_list_count, n) ? A.seed_list[s] : n;
       else if (A.front_list)
         s = front_seed(s, n, A.front_list, A.front_count, A.seed_surf, A.seed_keep != nullptr, A.counter);
@@ -931,7 +932,10 @@ __global__ void __launch_bounds__(LEARNED ? kFindMaxBlockLearned : 256, 2) k_fin
     // part in the selection and the seed goes to the second pass (its children all fit otherwise,
     // and keeping them all is what the full capacity does).
     constexpr bool RANK = !LEARNED && FEAT == 0;
-    int nch = (on && kind != 3) ? (kind == 0 ? (detect && !LEARNED ? npass : hl_n) : 1) : 0;
+    // (Passing hits beyond a lane's list are counted only where the list holds KC of them, so that a lane
+    // with more has overflowed; with k_max at or below the slots the list is all that a single pass
+    // would keep, and nothing beyond it may be offered.)
+    int nch = (on && kind != 3) ? (kind == 0 ? (!LEARNED && beyond ? npass : hl_n) : 1) : 0;
     auto child_key = [&](int h) {
       return kind == 0 ? pack_key(c.nh + 1, W.hl_tot[h][lane], slot << 2) | static_cast<unsigned>(h)
                        : pack_key(c.nh, c.chi2, (slot << 2) | kind);
@@ -947,9 +951,7 @@ __global__ void __launch_bounds__(LEARNED ? kFindMaxBlockLearned : 256, 2) k_fin
       const int all = __shfl_sync(kFull, cincl, in_grp ? gbase + KC - 1 : lane), tot = in_grp ? all : 0;
       ovf = detect && tot > KC;
       const int first = cincl - nch;  // number of this lane's first child
-      // A detecting pass with more slots than k_max counts passing hits that no list keeps: they make the
-      // seed overflow, but are not offered (their numbers stay empty below).
-      nch = ovf ? 0 : kind == 0 ? min(nch, hl_n) : nch;
+      if (ovf) nch = 0;
       const int most = static_cast<int>(__reduce_max_sync(kFull, ovf ? 0 : tot));
       unsigned long long* const kb = W.u.key + (in_grp ? grp * 2 * KC : 0);
       auto gather = [&](int c0, int c1, int at) {  // children numbered [c0, c1) to kb[at ...]
