@@ -57,11 +57,11 @@ FLOP_MLP_BWD = 2 * (64 * 64 + 64 * 64 + 64 * 14 + 64)
 # Both network kernels run their contractions on the tensor cores with every operand split into
 # three bf16 parts and six MMAs per product (FP32-faithful), so their roofline is the measured bf16
 # tensor peak / 6. MMA flops they issue per sample (M = 128 samples per tile, inputs padded to 16):
-# forward 6 x 2 (16 x 64 + 64 x 64); loss-gradient adds E2 W2 (6 x 2 x 64 x 64) and the weight-gradient
-# product [e2 | e1]^T [h1 | x | 1 | 0] (6 x 2 x 128 x 96).
+# forward 6 x 2 (16 x 64 + 64 x 64); loss-gradient adds E2 W2 (6 x 2 x 64 x 64) and the weight gradients'
+# MMAs of M = 128, N = 144, 80 and 64 (W2, b2) and 32, 16 and 16 (W1, b1), several products each.
 MLP_SPLIT_MMAS = 6
 MMA_MLP_FWD = MLP_SPLIT_MMAS * 2 * (16 * 64 + 64 * 64)
-MMA_MLP_GRAD = MMA_MLP_FWD + MLP_SPLIT_MMAS * 2 * (64 * 64 + 128 * 96)
+MMA_MLP_GRAD = MMA_MLP_FWD + MLP_SPLIT_MMAS * 2 * 64 * 64 + 2 * 128 * (144 + 80 + 64 + 32 + 16 + 16)
 # DRAM traffic of the finder measured by ncu (dram__bytes_read.sum + dram__bytes_write.sum of one
 # launch, or of adaptive capacity's two passes, per seed) on a smaller case of each workload (30
 # events of the 100-event workload, 40 of the barrel + disk workload; profiles/k_find_tracks_*),
@@ -72,15 +72,15 @@ FIND_SOURCES = ("paper_1906_02253_gb300/csrc/find.cu", "paper_1906_02253_gb300/c
                 "paper_1906_02253_gb300/csrc/find_learned.cu", "paper_1906_02253_gb300/csrc/kf_math.cuh",
                 "paper_1906_02253_gb300/csrc/find_launch.cuh", "paper_1906_02253_gb300/csrc/mlp.cuh",
                 "paper_1906_02253_gb300/build.py")
-FIND_PROFILE = {"sources_sha1": "e7656bf397b4a70bd709c2e54333c0d224d91176",
-                "dram_bytes_per_seed": {"fit_100ev_uneven_17layers_ms": (124858112 + 34387968) / 302063,
-                                        "find_200ev_barrel_disks_noise100": (231109376 + 69856768) / 211523,
+FIND_PROFILE = {"sources_sha1": "8415d6efe51744449eb06c7b05167dba52357bc5",
+                "dram_bytes_per_seed": {"fit_100ev_uneven_17layers_ms": (124911872 + 34346240) / 302063,
+                                        "find_200ev_barrel_disks_noise100": (231248640 + 70470656) / 211523,
                                         "find_200ev_barrel_disks_noise100_adaptive4":
-                                            (223592192 + 64325632 + 124954368 + 34751232) / 211523,
+                                            (223834880 + 64368896 + 125018880 + 34908672) / 211523,
                                         "find_200ev_barrel_disks_noise100_adaptive2":
-                                            (206157568 + 55670272 + 181676800 + 49921280) / 211523,
+                                            (206409472 + 55840512 + 182074112 + 50075136) / 211523,
                                         "find_200ev_barrel_disks_noise100_adaptive2_learned2_0.7":
-                                            (236084480 + 68200448 + 29479936 + 3928576) / 211523}}
+                                            (236923392 + 69208320 + 29477120 + 3939328) / 211523}}
 # Hit index: algorithmic HBM bytes per hit (read 8 B of (phi, z); write 8 B sorted, 4 B id, 16 B search
 # record) plus, per (event, surface), the bin offsets (4 B per bin + 1) and the phi sub-bin offsets (16 B per bin).
 INDEX_BYTES_PER_HIT = 36

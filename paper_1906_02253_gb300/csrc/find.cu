@@ -13,9 +13,13 @@ namespace kfgb {
 // |cot theta| / (1 + |cot theta|) run together, the central ones (most surfaces) first, so that the
 // last seeds are short. 24 classes (finder alone, measured on sorted seeds): 100 barrel + disk
 // events 4.57 -> 3.97 ms (8 classes 4.07, fully sorted 3.92, longest last 4.37, sorted in chunks of
-// 20 events 4.34), learned 4.38 -> 3.78, field map 1.75 -> 1.34. On barrel layers alone every
-// track crosses all of them and the order of the events serves the cache: sorted 10.4 against 9.8 ms,
-// so there the seeds stay in index order.
+// 20 events 4.34), learned 4.38 -> 3.78, field map 1.75 -> 1.34. The order spans the batch, so the longer
+// it is the more of the index is read from memory again; the present kernels against index order (a
+// workspace without the list), ns a seed on 60, 100, 300 and 600 events: two passes 7.4/8.4, 7.5/8.1,
+// 7.7/7.6, 7.7/7.6; one pass 9.4/9.9, 9.7/9.9, 9.9/9.8, 9.9/9.8; learned in two passes 7.0/7.8, 6.7/7.1,
+// 6.9/7.2, 6.7/6.7, in one 17.4/18.1, 17.9/18.1, 18.4/18.0, 18.6/18.0; field map 10.8/12.4, 11.2/12.8,
+// 11.5/12.3, 11.5/12.3. On barrel layers alone every track crosses all of them and the order of the
+// events serves the cache: sorted 10.4 against 9.8 ms, so there the seeds stay in index order.
 constexpr int kClasses = 24;
 __device__ __forceinline__ int seed_class(float theta) {
   float st, ct;

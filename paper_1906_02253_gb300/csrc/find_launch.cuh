@@ -34,18 +34,20 @@ struct FindArgs {
   float* state_out;
   float* cov_out;
   int* status_out;
-  // Workspace: the work counter (zeroed before each launch) and the fitted seed states.
+  // Workspace: the work counters (cleared before each call's kernels) and the fitted seed states.
   int* counter;
-  float* seed_state;  // [28][n_seeds]: p[6], C[21], chi2 (< 0: failed seed)
-  int* seed_surf;     // [n_seeds]: surface of the third seed hit
+  float* seed_state;  // p[6], C[21], chi2 (< 0: failed seed): for the finder one record of 28 words a seed
+                      // ([n_seeds][28]), for kf_seed_states its output ([28][n_seeds])
+  int* seed_surf;     // [n_seeds]: surface of the third seed hit (255: failed seed), a mark above it (find.cu)
   int* class_count;   // seeds of each direction class (the seed-state kernel counts them), or null
   int* front_list;    // seeds taken before the others (the seed-state kernel lists them), or null
   int* front_count;
-  // Adaptive capacity (plain finding): a first pass at a smaller capacity (detect = 1) finishes the
+  // Adaptive capacity: a first pass at a smaller capacity (detect = 1) finishes the
   // seeds whose children never outnumber its slots, which then have exactly the results of the
   // full capacity, and lists the others in ovf_list (*ovf_count of them) without writing their
   // outputs; the second pass takes its seeds from that list (seed_list, *seed_list_count). The
-  // first or only pass takes its seeds from the list ordered by direction, or in index order (null).
+  // first or only pass takes its seeds from the list ordered by direction (geometries with disks), or,
+  // with no list (null), the front list's first and then in index order.
   int detect;
   int* ovf_list;
   int* ovf_count;
@@ -68,8 +70,7 @@ struct FindPlan {
   size_t smem1, off_ovf;
 };
 
-// general: the geometry or the parameters use region steering, the material map, energy loss or
-// the parametrised field.
+// features: the options that the geometry and the parameters use (find_features).
 int plan_find(int n_seeds, const KfFindParams* p, int sms, int features, FindPlan* plan);
 inline int find_features(const DevGeom& G, const DevMat& M) {
   return (G.steer != 0 ? 1 : 0) | ((M.map_on != 0 || M.eloss > 0.f) ? 2 : 0) | (G.field_on != 0 ? 4 : 0);

@@ -60,9 +60,9 @@ __device__ __forceinline__ void parts_to_smem(unsigned char* t0, int row, int ha
 // relu(D1) -> the next A operand (in D1's columns; its lo part over the X tile, which the finished
 // MMA no longer needs); D2 = H W2^T; logit = b3 + sum_j W3[j] relu(D2[j] + b2[j]) on the CUDA cores.
 // Four groups per CTA (1024 threads at 64 registers, all 512 tensor-memory columns). 1,000,003 rows take
-// 53 us (192 TFLOP/s of the network's flops, six times that on the tensor cores: 60% of the measured
-// bf16 rate), where one chain per CTA, two CTAs per SM, took 115 us; the bound is the CUDA cores'
-// issue rate (splits, ReLU, output layer), then the tensor pipe.
+// 53 us (192 TFLOP/s of the network's flops, six times that on the tensor cores: 61% of the measured
+// bf16 rate), where one chain per CTA, two CTAs per SM, took 115 us. On 4 M rows issue is 59% active and
+// the tensor pipe 55%: what is left is a group's chain of barriers, MMA waits and operand stores.
 namespace fwd {
 constexpr int kGroups = 4;
 constexpr uint32_t W1_T = 2048, W2_T = 8192, H_T = 16384, X_T = 4096;  // bytes of one tile
@@ -177,8 +177,8 @@ __device__ __forceinline__ uint64_t dot16(const float* v, const float* w3, uint6
 
 // One MMA operand in shared memory: the descriptor of the first of its three tiles, whose size, layout
 // and advance per K = 16 step are compile-time constants, so that the thread that issues the MMAs
-// adds one constant to the descriptor's low word for each (with descriptors assembled per MMA,
-// by a thread picked by its index, an MMA took 56-85 cycles to issue, more than it ran).
+// adds one constant to the descriptor's low word for each (with descriptors assembled per MMA by a
+// thread picked by its index, the loss gradient of 2,000,003 rows took 604 us against 456).
 template <uint32_t LBO, uint32_t SBO, uint32_t STEP>
 struct Operand {
   uint32_t lo;
@@ -447,15 +447,14 @@ int launch_mlp_finder_scores(const float* params, const float* feats, int n, flo
 // the third MMA). With the parts side by side one gradient MMA does several of the six products:
 // per K = 16 step of dW2, [hi | mid] by [mid, hi, x hi] (M 128, N 144), [lo | 0] by [hi, x hi] (N 80)
 // and [hi | mid] by lo (N 64), into accumulators whose rows u and 64 + u, and columns c and 64 + c,
-// are added at the end; of dW1, [hi | mid] by [x hi, x mid], [lo | 0] by x hi, [hi | mid] by x lo. As
-// six products of M = 64 each (48 MMAs per layer, 40-60 cycles each: fetching the operands) they took
-// two thirds of the MMA time. The e tile (two do not fit) is one group's at a time, during its
+// are added at the end; of dW1, [hi | mid] by [x hi, x mid], [lo | 0] by x hi, [hi | mid] by x lo: half
+// the 48 MMAs per layer of six products of M = 64 each (2,000,003 rows 456 -> 415 us). The e tile (two do not fit) is one group's at a time, during its
 // gradient MMAs; the other group then runs its layers.
 // Tensor memory: per group D1, then h1, then e2 (parts_to_tmem) at 0, D2 then D3 at 96; Dg2 at 320,
 // Dg1 at 464.
-// 2,000,003 rows take 408 us (139 TFLOP/s of the network's flops), where one group per CTA took 895 us;
-// the bound is the tensor pipe fetching operands (a gradient MMA with an MN-major A of 128 rows takes 70
-// to 96 cycles). A step's 4,096 rows: the whole step 18 us against 98 us; their tile, prologue and epilogue
+// 2,000,003 rows take 407 us (140 TFLOP/s of the network's flops), where one group per CTA took 895 us.
+// On 4 M rows the tensor pipe is 42% active and issue 38%: the two groups' chains of six MMA round trips
+// a tile, one of them holding the e tile. A step's 4,096 rows: the whole step 18 us against 98 us; their tile, prologue and epilogue
 // are one chain (the old epilogue added 32 lanes to one shared-memory float, a CAS loop each).
 namespace grd {
 constexpr int kGroups = 2;
