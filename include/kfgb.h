@@ -175,8 +175,9 @@ typedef struct {
    * seeds whose children never outnumber those slots: keeping all of a step's children is what
    * k_max does then, so their results are those of the single pass. The other seeds are listed in
    * the workspace and found again, from their seed state, by a second pass at the full capacity.
-   * Ignored when no smaller compiled capacity exists or, with the learned proposal, when top_n
-   * exceeds the first pass's slots; KF_ERR_ARG outside [0, KF_MAX_K]. Pays where most seeds carry
+   * Where the first pass's slots hold k_max candidates it is the only pass. Ignored when no smaller
+   * compiled capacity exists or, with the learned proposal, when top_n exceeds the first pass's
+   * slots; KF_ERR_ARG outside [0, KF_MAX_K]. Pays where most seeds carry
    * few candidates (barrel + disk events with noise; the learned proposal's pruning). */
   int adaptive_capacity;
   /* Learned proposal ranking the window before the chi2 test (0 = off; 1 = on): the window is the

@@ -271,7 +271,7 @@ int plan_find(int n_seeds, const KfFindParams* p, int sms, int features, FindPla
   if (p->blocks_per_sm < 0) return KF_ERR_ARG;
   if (learned && p->block_threads > kFindMaxBlockLearned) return KF_ERR_CAPACITY;
   if (p->k_capacity < 0 || p->k_capacity > KF_MAX_K) return KF_ERR_ARG;
-  const int kc = pick_kc(std::max(learned ? std::max(p->k_max, p->top_n) : p->k_max, p->k_capacity));
+  int kc = pick_kc(std::max(learned ? std::max(p->k_max, p->top_n) : p->k_max, p->k_capacity));
   if (kc < 0) return KF_ERR_ARG;
   // Adaptive capacity: a first pass at the smallest compiled capacity >= the requested one, when
   // that is below the full capacity (and, with the learned proposal, holds top_n).
@@ -279,6 +279,12 @@ int plan_find(int n_seeds, const KfFindParams* p, int sms, int features, FindPla
   if (ac < 0 || ac > KF_MAX_K) return KF_ERR_ARG;
   int kc1 = ac > 0 ? pick_kc(ac) : 0;
   if (kc1 >= kc || (learned && p->top_n > kc1)) kc1 = 0;
+  // Slots for every candidate that is kept are all that a pass needs: such a first pass is the only one
+  // (and a detecting pass always has k_max above its slots).
+  if (kc1 >= p->k_max) {
+    kc = kc1;
+    kc1 = 0;
+  }
   // Resident blocks per SM for a block size (shared memory and registers), cached per (device,
   // capacity, mode, block size, lmax) so later calls, e.g. inside a stream capture, only launch.
   const int feat = compiled_features(learned, features);

@@ -514,13 +514,12 @@ __global__ void __launch_bounds__(LEARNED ? kFindMaxBlockLearned : 256, 2) k_fin
   WarpLearned<KC>& WL = *reinterpret_cast<WarpLearned<KC>*>(wbase + sizeof(WarpSmem<KC>) +
                                                             static_cast<size_t>(A.lmax - 3) * 32 * sizeof(int));
   const float* __restrict__ wmlp = A.mlp;  // network parameters (biases, output layer, normaliser)
-  // Capacity of a lane's list during the scan; a first pass of adaptive capacity (detect) keeps at
-  // most its own slots (a lane with more passing hits makes its seed overflow anyway). With the
+  // Capacity of a lane's list during the scan; a first pass of adaptive capacity (detect) keeps
+  // its own slots' number (a lane with more passing hits makes its seed overflow anyway). With the
   // learned proposal a first pass runs only when top_n fits its slots, so a lane's list holds
   // exactly its children.
   const int keep = LEARNED ? A.top_n : (A.detect ? min(A.k_max, KC) : A.k_max);
   const bool detect = A.detect != 0;
-  const bool beyond = detect && A.k_max > KC;  // passing hits beyond the lists count
   const bool margin_on = LEARNED && A.score_margin > 0.f;
   const bool window_rank = LEARNED && A.window_rank != 0;  // rank the window's box before the cut
   const int grp = lane / KC, slot = lane % KC;
@@ -932,10 +931,9 @@ __global__ void __launch_bounds__(LEARNED ? kFindMaxBlockLearned : 256, 2) k_fin
     // part in the selection and the seed goes to the second pass (its children all fit otherwise,
     // and keeping them all is what the full capacity does).
     constexpr bool RANK = !LEARNED && FEAT == 0;
-    // (Passing hits beyond a lane's list are counted only where the list holds KC of them, so that a lane
-    // with more has overflowed; with k_max at or below the slots the list is all that a single pass
-    // would keep, and nothing beyond it may be offered.)
-    int nch = (on && kind != 3) ? (kind == 0 ? (!LEARNED && beyond ? npass : hl_n) : 1) : 0;
+    // (A detecting pass has k_max > KC (plan_find), so its lists hold KC hits: a lane that counts more than
+    // its list holds has overflowed, and none beyond the list is offered.)
+    int nch = (on && kind != 3) ? (kind == 0 ? (detect && !LEARNED ? npass : hl_n) : 1) : 0;
     auto child_key = [&](int h) {
       return kind == 0 ? pack_key(c.nh + 1, W.hl_tot[h][lane], slot << 2) | static_cast<unsigned>(h)
                        : pack_key(c.nh, c.chi2, (slot << 2) | kind);
