@@ -72,15 +72,15 @@ FIND_SOURCES = ("paper_1906_02253_gb300/csrc/find.cu", "paper_1906_02253_gb300/c
                 "paper_1906_02253_gb300/csrc/find_learned.cu", "paper_1906_02253_gb300/csrc/kf_math.cuh",
                 "paper_1906_02253_gb300/csrc/find_launch.cuh", "paper_1906_02253_gb300/csrc/mlp.cuh",
                 "paper_1906_02253_gb300/build.py")
-FIND_PROFILE = {"sources_sha1": "8415d6efe51744449eb06c7b05167dba52357bc5",
-                "dram_bytes_per_seed": {"fit_100ev_uneven_17layers_ms": (124911872 + 34346240) / 302063,
-                                        "find_200ev_barrel_disks_noise100": (231248640 + 70470656) / 211523,
+FIND_PROFILE = {"sources_sha1": "dfd7403f314831b712ca87b484d2b9270fffb03e",
+                "dram_bytes_per_seed": {"fit_100ev_uneven_17layers_ms": (124845056 + 34342400) / 302063,
+                                        "find_200ev_barrel_disks_noise100": (230983168 + 70304256) / 211523,
                                         "find_200ev_barrel_disks_noise100_adaptive4":
-                                            (223834880 + 64368896 + 125018880 + 34908672) / 211523,
+                                            (223621376 + 64307712 + 124944128 + 34685696) / 211523,
                                         "find_200ev_barrel_disks_noise100_adaptive2":
-                                            (206409472 + 55840512 + 182074112 + 50075136) / 211523,
+                                            (206384896 + 56227328 + 181701376 + 49924352) / 211523,
                                         "find_200ev_barrel_disks_noise100_adaptive2_learned2_0.7":
-                                            (236923392 + 69208320 + 29477120 + 3939328) / 211523}}
+                                            (236838400 + 69143552 + 29475584 + 3916800) / 211523}}
 # Hit index: algorithmic HBM bytes per hit (read 8 B of (phi, z); write 8 B sorted, 4 B id, 16 B search
 # record) plus, per (event, surface), the bin offsets (4 B per bin + 1) and the phi sub-bin offsets (16 B per bin).
 INDEX_BYTES_PER_HIT = 36
